@@ -1,5 +1,6 @@
 // api.cu -- the C ABI of include/deoct.h: context, validation, and the host
 // orchestration of encoder, evaluator and DE kernels on the caller's stream.
+#include <algorithm>
 #include <cstring>
 #include <string>
 
@@ -149,14 +150,89 @@ EvalPlan single_eval_plan(const deoct_dataset* ds, const int32_t* idx, int64_t n
   return plan;
 }
 
-// evaluate one population on one (sub)set: counts must be zero beforehand
-static int eval_single(deoct_ctx* ctx, const deoct_dataset* ds, const int32_t* idx, int64_t n_sub,
-                       const uint32_t* nodes, uint32_t* counts, int P, int depth,
-                       cudaStream_t s) {
+// The bit-sliced evaluator's plan and shape for P trees with thresholds below
+// max_nu on one (sub)set; false: the other kernels take the launch.
+static bool slice_plan(const deoct_ctx* ctx, const deoct_dataset* ds, const int32_t* idx, int64_t n_sub, int P,
+                       int depth, int64_t max_nu, EvalPlan* plan, slc::SliceShape* sh) {
+  if (n_sub < 1 || P < 16) return false;  // (fewer trees run on the streaming kernel)
+  const int W = ds->rank_bytes, nb = slc::slice_bits(W, (uint32_t)max_nu);
+  if (!slc::slice_choose(ctx, depth, ds->F, ds->K, P, nb, slc::slice_tiles(n_sub), sh)) return false;
+  EvalConfig cfg;
+  cfg.S = 1024;
+  cfg.TG = sh->TG;
+  *plan = single_eval_plan(ds, idx, n_sub, nullptr, nullptr, P, cfg);
+  plan->single.nb = nb;
+  plan->single.W = W;
+  return true;
+}
+
+// Memory for the planes of a fit's (sub)set, which serve every generation: the
+// encoder's first buffer, which no fit reads and which is at least as large in a
+// context that encoded the set.  Without it (past that size, or past the context's
+// scratch limit) the evaluator transposes the ranks in every launch.
+// With enough tiles the planes hold the samples ordered by class (the order is
+// built in the encoder's second buffer), so that nearly every tile has one class.
+static int slice_planes_of_fit(deoct_ctx* ctx, const deoct_dataset* ds, const int32_t* idx, int64_t n_sub,
+                               EvalPlan* plan, cudaStream_t s) {
+  EvalProb& p = plan->single;
+  const int64_t tiles = slc::slice_tiles(n_sub);
+  const size_t bytes = slc::slice_plane_bytes(slc::slice_tiles(n_sub), ds->F, ds->K, p.nb);
+  if (bytes > std::max(ctx->scratch[SL_ENC_K0].bytes, 4 * (size_t)n_sub * ds->F)) return DEOCT_OK;
+  uint32_t* buf = nullptr;
+  if (scratch_get(ctx, SL_ENC_K0, bytes, (void**)&buf) != DEOCT_OK) {
+    clear_error();
+    return DEOCT_OK;
+  }
+  const size_t order_bytes = 3072 + sizeof(int32_t) * (size_t)n_sub;
+  unsigned char* order = nullptr;
+  if (ds->K > 1 && tiles >= 2 * ds->K &&
+      order_bytes <= std::max(ctx->scratch[SL_ENC_K1].bytes, 4 * (size_t)n_sub * ds->F)) {
+    if (scratch_get(ctx, SL_ENC_K1, order_bytes, (void**)&order) == DEOCT_OK) {
+      DEOCT_TRY(class_order(ctx, ds, idx, n_sub, reinterpret_cast<int32_t*>(order + 3072), order, s));
+      p.idx = reinterpret_cast<int32_t*>(order + 3072);
+      p.tma = p.lab_tma = 0;
+    } else {
+      clear_error();
+    }
+  }
+  p.planes = buf;
+  return slc::slice_planes(ctx, ds->rank_bytes, *plan, nullptr, 1, tiles, s);
+}
+
+// One evaluation on its own: trees from which the bit-sliced evaluator, which then
+// transposes every tile's ranks itself, is the faster one (GB300: 100 to 128 trees
+// 150 us against 145 at n = 1e6, F = 30, depth 3, 49 against 45 at n = 2e5, K = 10;
+// 256 trees 500 us against 790 at n = 2e6, depth 5; 1024 trees 4.5 ms against 10.2
+// at n = 1e7, depth 4).
+constexpr int kSliceOnce = 192;
+
+// Bound of an encoded set's ranks that needs no look at the device: its size, and
+// the rank width.  (Where a set breaks it the evaluator still counts right, slowly.)
+static int64_t width_bound(const deoct_dataset* ds) { return std::min<int64_t>(ds->n, ds->rank_bytes == 2 ? 65536 : kMaxN); }
+
+// evaluate one population on one (sub)set with the re-laid or the streaming kernel:
+// counts must be zero beforehand
+static int eval_ballot(deoct_ctx* ctx, const deoct_dataset* ds, const int32_t* idx, int64_t n_sub,
+                       const uint32_t* nodes, uint32_t* counts, int P, int depth, cudaStream_t s) {
   if (n_sub == 0) return DEOCT_OK;
   EvalConfig cfg = eval_choose_config(ctx, ds->rank_bytes, depth, ds->F, ds->K, P, n_sub, 1);
   EvalPlan plan = single_eval_plan(ds, idx, n_sub, nodes, counts, P, cfg);
   return eval_launch(ctx, ds->rank_bytes, depth, plan, cfg, s);
+}
+
+// the same with the evaluator that suits the shape
+static int eval_single(deoct_ctx* ctx, const deoct_dataset* ds, const int32_t* idx, int64_t n_sub,
+                       const uint32_t* nodes, uint32_t* counts, int P, int depth,
+                       cudaStream_t s) {
+  if (n_sub == 0) return DEOCT_OK;
+  EvalPlan sp;
+  slc::SliceShape sh;
+  if (P >= kSliceOnce && slice_plan(ctx, ds, idx, n_sub, P, depth, width_bound(ds), &sp, &sh)) {
+    sp.single.nodes = nodes;
+    sp.single.counts = counts;
+    return slc::slice_launch(ctx, depth, sp, sh, s);
+  }
+  return eval_ballot(ctx, ds, idx, n_sub, nodes, counts, P, depth, s);
 }
 
 // One evaluation of caller-given trees in a single launch: the evaluator packs
@@ -173,6 +249,17 @@ static int eval_single_fused(deoct_ctx* ctx, const deoct_dataset* ds, const int3
   uint32_t* base = nullptr;
   DEOCT_TRY(scratch_get(ctx, SL_EVAL_ACC, bytes, (void**)&base));
   if (grows) DEOCT_CUDA_TRY(cudaMemsetAsync(base, 0, ctx->scratch[SL_EVAL_ACC].bytes, s));
+  EvalPlan sp;
+  slc::SliceShape sh;
+  if (P >= kSliceOnce && slice_plan(ctx, ds, idx, n_sub, P, depth, width_bound(ds), &sp, &sh)) {
+    sp.single.a16 = a;
+    sp.single.th32 = theta;
+    sp.single.counts = base + 4;
+    sp.ticket = base;
+    sp.counts_out = counts_out;
+    sp.errors_out = errors_out;
+    return slc::slice_launch(ctx, depth, sp, sh, s);
+  }
   EvalConfig cfg = eval_choose_config(ctx, ds->rank_bytes, depth, ds->F, ds->K, P, n_sub, 1);
   EvalPlan plan = single_eval_plan(ds, idx, n_sub, nullptr, base + 4, P, cfg);
   plan.single.a16 = a;
@@ -245,14 +332,35 @@ static DEArgs de_args(const deoct_dataset* ds, const deoct_params* p, int64_t n_
 }
 
 // Algorithm 4 on one (sub)problem, device-resident: S^1, then G generations.
+// max_nu: the largest n_p of the set's features (0: read from the device here).
 int run_deoct(deoct_ctx* ctx, const deoct_dataset* ds, const int32_t* idx, int64_t n_sub,
               const deoct_params* p, uint64_t stream_id, const float* seeds, int S, float* pop,
-              double* fit, int32_t* best, cudaStream_t s) {
+              double* fit, int32_t* best, cudaStream_t s, uint32_t max_nu) {
   DEBuffers b;
   DEOCT_TRY(de_buffers(ctx, ds, p, &b));
   DEArgs a = de_args(ds, p, n_sub, stream_id, b, pop, fit, best, seeds, S, ctx->d_status);
   DEOCT_TRY(de_launch_init(ctx, a, s));
-  DEOCT_TRY(eval_single(ctx, ds, idx, n_sub, b.nodes, b.counts, p->pop, p->depth, s));
+  EvalPlan sp;
+  slc::SliceShape sh;
+  if (max_nu == 0) {
+    uint32_t* h = nullptr;
+    DEOCT_TRY(pinned_get(ctx, sizeof(uint32_t) * ds->F, (void**)&h));
+    DEOCT_CUDA_TRY(cudaMemcpyAsync(h, ds->n_unique, sizeof(uint32_t) * ds->F, cudaMemcpyDeviceToHost, s));
+    DEOCT_CUDA_TRY(cudaStreamSynchronize(s));
+    max_nu = *std::max_element(h, h + ds->F);
+  }
+  const bool sliced = slice_plan(ctx, ds, idx, n_sub, p->pop, p->depth, max_nu, &sp, &sh);
+  if (sliced) {
+    sp.single.nodes = b.nodes;
+    sp.single.counts = b.counts;
+    if (p->gens >= 1) DEOCT_TRY(slice_planes_of_fit(ctx, ds, idx, n_sub, &sp, s));
+    sh.raw = sp.single.planes == nullptr;
+  }
+  auto evaluate = [&](cudaStream_t st) {
+    return sliced ? slc::slice_launch(ctx, p->depth, sp, sh, st)
+                  : eval_ballot(ctx, ds, idx, n_sub, b.nodes, b.counts, p->pop, p->depth, st);
+  };
+  DEOCT_TRY(evaluate(s));
   // The generation number lives on the device (set to 1 by the init kernel and
   // advanced by every trial step), so every generation is the same pair of
   // launches: captured once as a CUDA graph and replayed G times.  With
@@ -262,7 +370,7 @@ int run_deoct(deoct_ctx* ctx, const deoct_dataset* ds, const int32_t* idx, int64
   if (p->gens < 1) return DEOCT_OK;
   if (ctx->timing || p->gens < 3) {
     for (int g = 1; g <= p->gens; ++g) {
-      DEOCT_TRY(eval_single(ctx, ds, idx, n_sub, b.nodes, b.counts, p->pop, p->depth, s));
+      DEOCT_TRY(evaluate(s));
       DEOCT_TRY(de_launch_step(ctx, a, 0, DE_SELECT | DE_TRIAL | DE_GEN_DEVICE, s));
     }
     return DEOCT_OK;
@@ -273,7 +381,7 @@ int run_deoct(deoct_ctx* ctx, const deoct_dataset* ds, const int32_t* idx, int64
   cudaGraph_t graph = nullptr;
   cudaGraphExec_t exec = nullptr;
   DEOCT_CUDA_TRY(cudaStreamBeginCapture(ctx->cap_stream, cudaStreamCaptureModeThreadLocal));
-  int rc = eval_single(ctx, ds, idx, n_sub, b.nodes, b.counts, p->pop, p->depth, ctx->cap_stream);
+  int rc = evaluate(ctx->cap_stream);
   if (rc == DEOCT_OK) rc = de_launch_step(ctx, a, 0, DE_SELECT | DE_TRIAL | DE_GEN_DEVICE, ctx->cap_stream);
   cudaError_t ce = cudaStreamEndCapture(ctx->cap_stream, &graph);
   const uint64_t per_launch = ctx->launches - l0, per_eval = ctx->eval_launches - e0;
@@ -695,7 +803,7 @@ int deoct_fit_subtree(deoct_ctx* ctx, const deoct_dataset* ds, const int32_t* sa
   int32_t* best = nullptr;
   DEOCT_TRY(scratch_get(ctx, SL_FIT, P * sizeof(double), (void**)&fit));
   DEOCT_TRY(scratch_get(ctx, SL_BEST, 64, (void**)&best));
-  DEOCT_TRY(run_deoct(ctx, ds, sample_idx, n_sub, params, stream_id, seeds, S, pop, fit, best, s));
+  DEOCT_TRY(run_deoct(ctx, ds, sample_idx, n_sub, params, stream_id, seeds, S, pop, fit, best, s, 0));
   // decoded best tree -> host
   unsigned char* dres = nullptr;
   const size_t res_bytes = 8 + B * 2 + B * 4 + 16;

@@ -27,6 +27,13 @@ struct EvalProb {
   // is unused then
   const uint16_t* a16 = nullptr;
   const uint32_t* th32 = nullptr;
+  // bit-sliced evaluator: the problem's planes (tile blocks of F nb + K rows of 32
+  // words; nullptr: the evaluator transposes the ranks itself), the planes a feature
+  // has (0: not set up for it), the rank width in bytes, and the problem's first tile
+  // among those of the launch's problems
+  const uint32_t* planes = nullptr;
+  int64_t ptile0 = 0;
+  int32_t nb = 0, W = 0;
 };
 // A job is one tree group of one problem; its tiles are contiguous in the
 // flattened tile order that the persistent CTAs split evenly.
@@ -70,6 +77,26 @@ struct EvalPlan {
 
 int eval_launch(deoct_ctx* ctx, int W, int D, const EvalPlan& plan, const EvalConfig& cfg,
                 cudaStream_t stream);
+
+// The bit-sliced evaluator (eval_slice.cuh).  slice_choose says whether it takes
+// a launch (D <= 5, the thermometer rows of F features fit shared memory, no
+// forced launch shape) and with what shape; slice_planes builds the planes of a
+// plan's problems, slice_launch evaluates them.
+namespace slc {
+struct SliceShape {
+  int TG = 0, nd = 0, rows = 0, rec_bytes = 0;
+  bool raw = true;  // no planes in memory (all of a launch's problems have them, or none)
+};
+int64_t slice_tiles(int64_t count);                // tiles of 1024 samples
+size_t slice_plane_bytes(int64_t tiles, int F, int K, int nb);
+int slice_bits(int W, uint32_t max_nu);            // planes that hold every theta < max_nu
+// nb: planes per feature; tiles: of all problems, for one tree group
+bool slice_choose(const deoct_ctx* ctx, int D, int F, int K, int P, int nb, int64_t tiles, SliceShape* out);
+int slice_planes(deoct_ctx* ctx, int W, const EvalPlan& plan, const EvalProb* d_probs, int nprob, int64_t tiles,
+                 cudaStream_t s);
+int slice_launch(deoct_ctx* ctx, int D, const EvalPlan& plan, const SliceShape& shape, cudaStream_t s);
+}  // namespace slc
+
 // CTAs of a re-laid-kernel shape resident on one SM (shared memory and registers;
 // 0 when the shape does not fit or runs on the streaming kernel).
 int eval_ctas_per_sm(const deoct_ctx* ctx, int W, int D, int F, int K, const EvalConfig& c);
@@ -186,6 +213,9 @@ int radix_sort_segments(deoct_ctx* ctx, uint32_t* k0, uint32_t* v0, uint32_t* k1
 int engine_generations(deoct_engine* e, const void* owner, int W, int Dt, const DEArgs& a, int G,
                        const std::vector<DEProb>& dp, const std::vector<EvalProb>& ep);
 
+// the columns of a (sub)set ordered by class (mh.cu); tmp: 3072 bytes of device memory
+int class_order(deoct_ctx* ctx, const deoct_dataset* ds, const int32_t* idx, int64_t n, int32_t* order, void* tmp,
+                cudaStream_t s);
 size_t fit_scratch_bound(const deoct_ctx* ctx, int64_t n, int F, int K, int W, const deoct_params* prm);
 int mh_run(deoct_ctx* ctx, const deoct_dataset* ds, const deoct_params* prm, uint16_t* a_out,
            uint32_t* th_out, uint8_t* leaf_class_out, int32_t* kind_out, double* node_fit_out,

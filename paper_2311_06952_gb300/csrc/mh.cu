@@ -29,7 +29,7 @@ namespace deoct {
 
 int run_deoct(deoct_ctx* ctx, const deoct_dataset* ds, const int32_t* idx, int64_t n_sub,
               const deoct_params* p, uint64_t stream_id, const float* seeds, int S, float* pop,
-              double* fit, int32_t* best, cudaStream_t s);
+              double* fit, int32_t* best, cudaStream_t s, uint32_t max_nu);
 
 namespace {
 
@@ -82,29 +82,118 @@ __global__ void route_level_kernel(int32_t* __restrict__ node_of, const RT* __re
   node_of[i] = 2 * t + (r < th ? 0 : 1);
 }
 
-// samples of solved nodes -> contiguous segments (order inside a segment is
-// arbitrary: every consumer is order-independent)
-__global__ void compact_kernel(const int32_t* __restrict__ node_of, int64_t n, int32_t base,
-                               int32_t nnodes, const int32_t* __restrict__ slot_of,
-                               const int64_t* __restrict__ seg_off, int32_t* __restrict__ cursor,
-                               int32_t* __restrict__ idx_out, int32_t* __restrict__ pos_slot) {
-  int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  int m = -1;
-  if (i < n) {
-    int k = node_of[i] - base;
-    if (k >= 0 && k < nnodes) m = slot_of[k];
-  }
+// Samples grouped by key (class fastest: key = group K + class): each key's
+// samples go to consecutive positions from off[key], in any order -- every
+// consumer is order-independent, but the evaluator's tiles are cheaper when a
+// tile's samples have one class (eval_slice.cuh).  A block counts the keys of its
+// 4096 samples in shared memory, reserves each key's positions with one atomic,
+// then places them.  kSmem = false: too many keys for shared memory, one global
+// atomic per warp and key.
+constexpr int kGroupThreads = 256, kGroupItems = 16;
+constexpr int kGroupKeys = 8192;  // most keys counted in shared memory
+
+template <bool kSmem, typename KeyOf, typename Put>
+__device__ __forceinline__ void group_samples(int64_t n, int nkeys, const int64_t* __restrict__ off,
+                                              int32_t* __restrict__ cursor, KeyOf key_of, Put put) {
+  extern __shared__ int32_t gk[];  // counts, then next positions, of the block's keys
   const int lane = threadIdx.x & 31;
-  const uint32_t peers = __match_any_sync(0xFFFFFFFFu, m);
-  const int leader = __ffs(peers) - 1;
-  int basepos = 0;
-  if (m >= 0 && lane == leader) basepos = atomicAdd(&cursor[m], __popc(peers));
-  basepos = __shfl_sync(0xFFFFFFFFu, basepos, leader);
-  if (m >= 0) {
-    int64_t pos = seg_off[m] + basepos + __popc(peers & ((1u << lane) - 1u));
-    idx_out[pos] = (int32_t)i;
-    pos_slot[pos] = m;
+  const int64_t base = (int64_t)blockIdx.x * (kGroupThreads * kGroupItems);
+  int key[kGroupItems];
+#pragma unroll
+  for (int it = 0; it < kGroupItems; ++it) {
+    const int64_t i = base + it * kGroupThreads + threadIdx.x;
+    key[it] = i < n ? key_of(i) : -1;
   }
+  if (kSmem) {
+    for (int e = threadIdx.x; e < nkeys; e += kGroupThreads) gk[e] = 0;
+    __syncthreads();
+#pragma unroll
+    for (int it = 0; it < kGroupItems; ++it) {
+      const uint32_t peers = __match_any_sync(0xFFFFFFFFu, key[it]);
+      if (key[it] >= 0 && (__ffs(peers) - 1) == lane) atomicAdd(&gk[key[it]], __popc(peers));
+    }
+    __syncthreads();
+    for (int e = threadIdx.x; e < nkeys; e += kGroupThreads) {
+      const int c = gk[e];
+      if (c) gk[e] = atomicAdd(&cursor[e], c);
+    }
+    __syncthreads();
+  }
+#pragma unroll
+  for (int it = 0; it < kGroupItems; ++it) {
+    const int k = key[it];
+    const uint32_t peers = __match_any_sync(0xFFFFFFFFu, k);
+    const int leader = __ffs(peers) - 1;
+    int pos = 0;
+    if (k >= 0 && lane == leader) pos = atomicAdd(kSmem ? &gk[k] : &cursor[k], __popc(peers));
+    pos = __shfl_sync(0xFFFFFFFFu, pos, leader);
+    if (k >= 0) put(off[k] + pos + __popc(peers & ((1u << lane) - 1u)), base + it * kGroupThreads + threadIdx.x, k);
+  }
+}
+
+// samples of solved nodes -> contiguous segments, by class inside a segment
+template <bool kSmem>
+__global__ void __launch_bounds__(kGroupThreads) compact_kernel(
+    const int32_t* __restrict__ node_of, const uint8_t* __restrict__ labels, int64_t n, int32_t base, int32_t nnodes,
+    int K, int nkeys, const int32_t* __restrict__ slot_of, const int64_t* __restrict__ key_off,
+    int32_t* __restrict__ cursor, int32_t* __restrict__ idx_out, int32_t* __restrict__ pos_slot) {
+  group_samples<kSmem>(
+      n, nkeys, key_off, cursor,
+      [&](int64_t i) {
+        const int k = node_of[i] - base;
+        if (k < 0 || k >= nnodes) return -1;
+        const int m = slot_of[k], y = labels[i];
+        return m >= 0 && y < K ? m * K + y : -1;
+      },
+      [&](int64_t pos, int64_t i, int key) {
+        idx_out[pos] = (int32_t)i;
+        pos_slot[pos] = key / K;
+      });
+}
+
+// Class histogram of a (sub)set (K + 1 bins: labels past K count as class K), and
+// its columns ordered by class.
+__device__ __forceinline__ int class_of(const uint8_t* labels, const int32_t* idx, int64_t ncols, int K, int64_t i) {
+  int64_t col = i;
+  if (idx) {
+    col = idx[i];
+    if ((uint64_t)col >= (uint64_t)ncols) col = 0;  // flagged where the ranks are read
+  }
+  const int y = labels[col];
+  return y < K ? y : K;
+}
+__global__ void class_hist_kernel(const uint8_t* __restrict__ labels, const int32_t* __restrict__ idx, int64_t ncols,
+                                  int64_t n, int K, int32_t* __restrict__ hist) {
+  __shared__ int32_t h[kMaxK + 1];
+  for (int e = threadIdx.x; e <= K; e += blockDim.x) h[e] = 0;
+  __syncthreads();
+  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
+    atomicAdd(&h[class_of(labels, idx, ncols, K, i)], 1);
+  __syncthreads();
+  for (int e = threadIdx.x; e <= K; e += blockDim.x)
+    if (h[e]) atomicAdd(&hist[e], h[e]);
+}
+// exclusive scan of at most 256 counts -> offsets; the counts become cursors (zero)
+__global__ void __launch_bounds__(256) class_offsets_kernel(int32_t* __restrict__ hist, int K, int64_t* __restrict__ off) {
+  __shared__ int32_t h[kMaxK + 1];
+  const int t = threadIdx.x;
+  if (t <= K) {
+    h[t] = hist[t];
+    hist[t] = 0;
+  }
+  __syncthreads();
+  if (t <= K) {
+    int64_t s = 0;
+    for (int k = 0; k < t; ++k) s += h[k];
+    off[t] = s;
+  }
+}
+__global__ void __launch_bounds__(kGroupThreads) class_order_kernel(
+    const uint8_t* __restrict__ labels, const int32_t* __restrict__ idx, int64_t ncols, int64_t n, int K,
+    const int64_t* __restrict__ off, int32_t* __restrict__ cursor, int32_t* __restrict__ out) {
+  group_samples<true>(
+      n, K + 1, off, cursor, [&](int64_t i) { return class_of(labels, idx, ncols, K, i); },
+      [&](int64_t pos, int64_t i, int) { out[pos] = idx ? idx[i] : (int32_t)i; });
 }
 
 // compacted rank rows and labels (padding: rank 0, label 0xFF)
@@ -448,6 +537,41 @@ struct BatchedEval {
   EvalPlan plan;
 };
 
+// The bit-sliced evaluator's shape for a level's problems, with memory for their
+// planes in the encoder's first buffer (4 n F bytes in a context that encoded the
+// set, and no fit reads it; without it the evaluator transposes the ranks in
+// every launch).  False: the other kernels evaluate the level.
+bool level_planes(deoct_ctx* ctx, const deoct_dataset* ds, BatchedEval* be, int P, int Dt, uint32_t max_nu,
+                  slc::SliceShape* sh) {
+  if (P < 16) return false;
+  const int nb = slc::slice_bits(ds->rank_bytes, max_nu);
+  int64_t tiles = 0;
+  for (EvalProb& e : be->probs) {
+    e.ptile0 = tiles;
+    tiles += slc::slice_tiles(e.count);
+  }
+  // nodes of a few dozen samples leave most of a tile empty (n = 4000 over 64 nodes:
+  // 12.9 ms a fit against 11.9 with the re-laid kernel; n = 16000 over 32: 11.8 against 13.4)
+  int64_t samples = 0;
+  for (const EvalProb& e : be->probs) samples += e.count;
+  if (be->probs.size() > 1 && samples < 384 * tiles) return false;
+  if (!slc::slice_choose(ctx, Dt, ds->F, ds->K, P, nb, tiles, sh)) return false;
+  for (EvalProb& e : be->probs) {
+    e.nb = nb;
+    e.W = ds->rank_bytes;
+  }
+  const size_t bytes = slc::slice_plane_bytes(tiles, ds->F, ds->K, nb);
+  uint32_t* planes = nullptr;
+  if (bytes > std::max(ctx->scratch[SL_ENC_K0].bytes, 4 * (size_t)ds->n * ds->F)) return true;
+  if (scratch_get(ctx, SL_ENC_K0, bytes, (void**)&planes) != DEOCT_OK) {  // past the scratch limit
+    clear_error();
+    return true;
+  }
+  sh->raw = false;
+  for (EvalProb& e : be->probs) e.planes = planes + slc::slice_plane_bytes(e.ptile0, ds->F, ds->K, nb) / 4;
+  return true;
+}
+
 int build_plan(deoct_ctx* ctx, BatchedEval* be, const EvalConfig& cfg, int F, int K, int P,
                cudaStream_t s) {
   std::vector<int64_t> counts(be->probs.size());
@@ -511,7 +635,7 @@ uint64_t tune_key(int W, int D, int F, int K, int P, int64_t npad, int M) {
 
 // Batched DEOCT for all segments of a level: one evaluator launch and one DE
 // step launch per generation, replayed from a captured CUDA graph.
-int de_batched(deoct_ctx* ctx, const deoct_dataset* ds, const Compacted& c,
+int de_batched(deoct_ctx* ctx, const deoct_dataset* ds, const Compacted& c, uint32_t max_nu,
                const std::vector<int>& node_ids, int Dt, const deoct_params* prm,
                const float* d_seeds, int S, std::vector<uint16_t>* ra, std::vector<uint32_t>* rth,
                std::vector<double>* rf, cudaStream_t s) {
@@ -569,6 +693,8 @@ int de_batched(deoct_ctx* ctx, const deoct_dataset* ds, const Compacted& c,
     e.tma = 1;
     e.lab_tma = (reinterpret_cast<uintptr_t>(c.clabels + e.start) % 16 == 0) ? 1 : 0;
   }
+  slc::SliceShape sh;
+  const bool sliced = level_planes(ctx, ds, &be, P, Dt, max_nu, &sh);
   DEProb* ddp = nullptr;
   EvalProb* dep = nullptr;
   DEOCT_TRY(upload(ctx, SL_DE_PROBS, dp, &ddp, s));
@@ -588,13 +714,25 @@ int de_batched(deoct_ctx* ctx, const deoct_dataset* ds, const Compacted& c,
   a.Kmax = K;
   a.status = ctx->d_status;
   DEOCT_TRY(de_launch_init(ctx, a, s));
+  EvalConfig scfg;
+  scfg.S = 1024;
+  scfg.TG = sh.TG;
+  if (sliced && be.probs[0].planes) {
+    be.plan.Fmax = F;
+    int64_t tiles = 0;
+    for (const EvalProb& e : be.probs) tiles += slc::slice_tiles(e.count);
+    DEOCT_TRY(slc::slice_planes(ctx, W, be.plan, dep, M, tiles, s));
+  }
+  auto evaluate = [&](const EvalConfig& cfg, cudaStream_t st) {
+    return sliced ? slc::slice_launch(ctx, Dt, be.plan, sh, st) : eval_launch(ctx, W, Dt, be.plan, cfg, st);
+  };
 
   if (ctx->engine) {
     // S^1 and the first trials here, then the G generations in the engine's
     // launches shared with other jobs
-    EvalConfig cfg = eval_choose_config(ctx, W, Dt, F, K, P, std::max<int64_t>(1, nsum_of(c, M)), M);
+    EvalConfig cfg = sliced ? scfg : eval_choose_config(ctx, W, Dt, F, K, P, std::max<int64_t>(1, nsum_of(c, M)), M);
     DEOCT_TRY(build_plan(ctx, &be, cfg, F, K, P, s));
-    DEOCT_TRY(eval_launch(ctx, W, Dt, be.plan, cfg, s));
+    DEOCT_TRY(evaluate(cfg, s));
     DEOCT_TRY(de_launch_step(ctx, a, 0, DE_FIRST | DE_GEN_DEVICE | (prm->gens >= 1 ? DE_TRIAL : 0), s));
     DEOCT_CUDA_TRY(cudaStreamSynchronize(s));
     if (prm->gens >= 1) DEOCT_TRY(engine_generations(ctx->engine, ctx, W, Dt, a, prm->gens, dp, be.probs));
@@ -621,7 +759,7 @@ int de_batched(deoct_ctx* ctx, const deoct_dataset* ds, const Compacted& c,
   // from 2e10 tree-sample evaluations (~20 ms on GB300) on; smaller levels take the
   // chooser's shape
   const bool worth = (double)nsum * P * (prm->gens + 1) >= 2e10;
-  if (!have && !forced && worth) {
+  if (!sliced && !have && !forced && worth) {
     // candidates around the heuristic; each runs the real evaluation of S^1
     std::vector<EvalConfig> cands{cfg};  // the heuristic's own shape first
     for (int S : {256, 512, 1024, 2048})
@@ -714,10 +852,11 @@ int de_batched(deoct_ctx* ctx, const deoct_dataset* ds, const Compacted& c,
     for (int m = 0; m < M; ++m)
       DEOCT_CUDA_TRY(cudaMemsetAsync(dp[m].counts, 0, (size_t)P * L * K * 4, s));
   }
+  if (sliced) cfg = scfg;
   DEOCT_TRY(build_plan(ctx, &be, cfg, F, K, P, s));
 
   // ---- S^1, then G generations from one captured graph ---------------------
-  DEOCT_TRY(eval_launch(ctx, W, Dt, be.plan, cfg, s));
+  DEOCT_TRY(evaluate(cfg, s));
   DEOCT_TRY(de_launch_step(ctx, a, 0, DE_FIRST | DE_GEN_DEVICE | (prm->gens >= 1 ? DE_TRIAL : 0), s));
   if (prm->gens >= 1) {
     if (!ctx->cap_stream)
@@ -726,7 +865,7 @@ int de_batched(deoct_ctx* ctx, const deoct_dataset* ds, const Compacted& c,
     cudaGraphExec_t exec = nullptr;
     const uint64_t l0 = ctx->launches, e0n = ctx->eval_launches;
     DEOCT_CUDA_TRY(cudaStreamBeginCapture(ctx->cap_stream, cudaStreamCaptureModeThreadLocal));
-    int rc = eval_launch(ctx, W, Dt, be.plan, cfg, ctx->cap_stream);
+    int rc = evaluate(cfg, ctx->cap_stream);
     if (rc == DEOCT_OK)
       rc = de_launch_step(ctx, a, 0, DE_SELECT | DE_TRIAL | DE_GEN_DEVICE, ctx->cap_stream);
     cudaError_t ce = cudaStreamEndCapture(ctx->cap_stream, &graph);
@@ -760,7 +899,7 @@ int de_batched(deoct_ctx* ctx, const deoct_dataset* ds, const Compacted& c,
 }
 
 // Plain form: one DEOCT (own launches) per node segment.
-int de_plain(deoct_ctx* ctx, const deoct_dataset* ds, const Compacted& c,
+int de_plain(deoct_ctx* ctx, const deoct_dataset* ds, const Compacted& c, uint32_t max_nu,
              const std::vector<int>& node_ids, int Dt, const deoct_params* prm, const float* d_seeds,
              int S, std::vector<uint16_t>* ra, std::vector<uint32_t>* rth, std::vector<double>* rf,
              cudaStream_t s) {
@@ -786,7 +925,7 @@ int de_plain(deoct_ctx* ctx, const deoct_dataset* ds, const Compacted& c,
     deoct_dataset v = segment_view(ds, c, m);
     const float* sd = (d_seeds && S > 0) ? d_seeds + (size_t)m * S * 2 * B : nullptr;
     DEOCT_TRY(run_deoct(ctx, &v, nullptr, v.n, &dp, (uint64_t)node_ids[m], sd, sd ? S : 0, pop, fit,
-                        best, s));
+                        best, s, max_nu));
     DEOCT_TRY(launch_best_extract(ctx, pop, fit, best, Dt, ds->F, ds->n_unique, da, dth, df, s));
     std::vector<double> hf;
     std::vector<uint32_t> hth;
@@ -1013,6 +1152,23 @@ int launch_level_hist(deoct_ctx* ctx, const deoct_dataset* ds, const int32_t* no
 
 }  // namespace
 
+// The columns of a (sub)set ordered by class -> order [n] (device); tmp: 3072 bytes
+// of device memory.
+int class_order(deoct_ctx* ctx, const deoct_dataset* ds, const int32_t* idx, int64_t n, int32_t* order, void* tmp,
+                cudaStream_t s) {
+  int64_t* off = static_cast<int64_t*>(tmp);
+  int32_t* cur = reinterpret_cast<int32_t*>(off + kMaxK + 1);
+  DEOCT_CUDA_TRY(cudaMemsetAsync(cur, 0, sizeof(int32_t) * (ds->K + 1), s));
+  const int hgrid = (int)std::min<int64_t>((n + 1023) / 1024, (int64_t)ctx->num_sms * 4);
+  class_hist_kernel<<<hgrid, 256, 0, s>>>(ds->labels, idx, ds->n, n, ds->K, cur);
+  class_offsets_kernel<<<1, 256, 0, s>>>(cur, ds->K, off);
+  const int per = kGroupThreads * kGroupItems;
+  class_order_kernel<<<(unsigned)((n + per - 1) / per), kGroupThreads, sizeof(int32_t) * (ds->K + 1), s>>>(
+      ds->labels, idx, ds->n, n, ds->K, off, cur, order);
+  count_launch(ctx, 3);
+  return check_launch("class order kernels");
+}
+
 // Algorithm 2, level by level.
 int mh_run(deoct_ctx* ctx, const deoct_dataset* ds, const deoct_params* prm, uint16_t* a_out,
            uint32_t* th_out, uint8_t* leaf_class_out, int32_t* kind_out, double* node_fit_out,
@@ -1034,6 +1190,7 @@ int mh_run(deoct_ctx* ctx, const deoct_dataset* ds, const deoct_params* prm, uin
   std::vector<int> full_a;
   std::vector<uint32_t> full_th, nu_host;
   DEOCT_TRY(download(ctx, ds->n_unique, (size_t)ds->F, &nu_host, s));
+  const uint32_t max_nu = *std::max_element(nu_host.begin(), nu_host.end());
   if ((prm->flags & DEOCT_DE_SEEDS) && D >= 2 && H >= 2) {
     deoct_params fp = *prm;
     fp.depth = D;
@@ -1043,7 +1200,7 @@ int mh_run(deoct_ctx* ctx, const deoct_dataset* ds, const deoct_params* prm, uin
     DEOCT_TRY(scratch_get(ctx, SL_POP, (size_t)prm->pop * 2 * B * 4, (void**)&pop));
     DEOCT_TRY(scratch_get(ctx, SL_FIT, (size_t)prm->pop * 8, (void**)&fit));
     DEOCT_TRY(scratch_get(ctx, SL_BEST, 64, (void**)&best));
-    DEOCT_TRY(run_deoct(ctx, ds, nullptr, n, &fp, 0, nullptr, 0, pop, fit, best, s));
+    DEOCT_TRY(run_deoct(ctx, ds, nullptr, n, &fp, 0, nullptr, 0, pop, fit, best, s, max_nu));
     unsigned char* dres;
     DEOCT_TRY(scratch_get(ctx, SL_D1_RESULT, (size_t)B * 6 + 64, (void**)&dres));
     double* df = reinterpret_cast<double*>(dres);
@@ -1088,17 +1245,32 @@ int mh_run(deoct_ctx* ctx, const deoct_dataset* ds, const deoct_params* prm, uin
     if (M > 0) {
       c.npad = std::max<int64_t>(off, kSegAlign);
       const int Dt = std::min(H, D - d);
+      // first position of every (node, class) of the level
+      const int nkeys = M * K;
+      std::vector<int64_t> key_off(nkeys);
+      for (int m = 0; m < M; ++m) {
+        int64_t at = c.seg_off[m];
+        for (int y = 0; y < K; ++y) {
+          key_off[(size_t)m * K + y] = at;
+          at += hh[(size_t)(solved[m] - base) * K + y];
+        }
+      }
       int32_t* dslot;
-      int64_t* dseg;
+      int64_t* dkey;
       int32_t* dcur;
       DEOCT_TRY(upload(ctx, SL_MH_SEG, slot_of, &dslot, s));
-      DEOCT_TRY(upload(ctx, SL_MH_STATS, c.seg_off, &dseg, s));
-      DEOCT_TRY(scratch_get(ctx, SL_MH_CURSOR, sizeof(int32_t) * M, (void**)&dcur));
-      DEOCT_CUDA_TRY(cudaMemsetAsync(dcur, 0, sizeof(int32_t) * M, s));
+      DEOCT_TRY(upload(ctx, SL_MH_STATS, key_off, &dkey, s));
+      DEOCT_TRY(scratch_get(ctx, SL_MH_CURSOR, sizeof(int32_t) * nkeys, (void**)&dcur));
+      DEOCT_CUDA_TRY(cudaMemsetAsync(dcur, 0, sizeof(int32_t) * nkeys, s));
       DEOCT_TRY(launch_fill(ctx, c.idx, c.npad, -1, s));
       DEOCT_TRY(launch_fill(ctx, c.pos_slot, c.npad, -1, s));
-      compact_kernel<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(node_of, n, base, nn, dslot, dseg, dcur,
-                                                                c.idx, c.pos_slot);
+      const unsigned cgrid = (unsigned)((n + kGroupThreads * kGroupItems - 1) / (kGroupThreads * kGroupItems));
+      if (nkeys <= kGroupKeys)
+        compact_kernel<true><<<cgrid, kGroupThreads, sizeof(int32_t) * nkeys, s>>>(
+            node_of, ds->labels, n, base, nn, K, nkeys, dslot, dkey, dcur, c.idx, c.pos_slot);
+      else
+        compact_kernel<false><<<cgrid, kGroupThreads, 0, s>>>(node_of, ds->labels, n, base, nn, K, nkeys, dslot, dkey,
+                                                             dcur, c.idx, c.pos_slot);
       count_launch(ctx);
       DEOCT_TRY(check_launch("compact_kernel"));
       DEOCT_TRY(gather_compacted(ctx, ds, &c, s));
@@ -1135,8 +1307,8 @@ int mh_run(deoct_ctx* ctx, const deoct_dataset* ds, const deoct_params* prm, uin
           }
           DEOCT_TRY(upload(ctx, SL_MH_SEEDS, all, &seeds, s));
         }
-        if (batched) DEOCT_TRY(de_batched(ctx, ds, c, solved, Dt, prm, seeds, S, &ra, &rth, &rf, s));
-        else DEOCT_TRY(de_plain(ctx, ds, c, solved, Dt, prm, seeds, S, &ra, &rth, &rf, s));
+        if (batched) DEOCT_TRY(de_batched(ctx, ds, c, max_nu, solved, Dt, prm, seeds, S, &ra, &rth, &rf, s));
+        else DEOCT_TRY(de_plain(ctx, ds, c, max_nu, solved, Dt, prm, seeds, S, &ra, &rth, &rf, s));
       } else {
         kd = 1;
         if (batched) {
@@ -1224,9 +1396,9 @@ size_t fit_scratch_bound(const deoct_ctx* ctx, int64_t n, int F, int K, int W, c
   // warm starts work on (node, subtree node) pairs: at most nn * L / 2 of them
   const int Dt = std::min(H, D), B = (1 << Dt) - 1, L = 1 << Dt;
   const double pairs = (double)nn * std::max(1, L / 2);
-  need(SL_MH_STATS, std::max(8.0 * pairs, 4.0 * pairs * K));
+  need(SL_MH_STATS, std::max({8.0 * pairs, 4.0 * pairs * K, 8.0 * nn * K}));
   need(SL_MH_SEG, std::max(4.0 * pairs, 8.0 * 255));
-  need(SL_MH_CURSOR, std::max(4.0 * pairs, 8.0 * 255));
+  need(SL_MH_CURSOR, std::max({4.0 * pairs, 4.0 * nn * K, 8.0 * 255}));
   need(SL_MH_D1BEST, 12.0 * 255 * F + 64);
   need(SL_D1_RESULT, std::max(16.0 * std::max<double>(pairs, 255) + 64, 6.0 * (Lf - 1) + 64));
   const double per = (double)P * 2 * B * 4 * 2 + (double)P * 8 * 2 + 16 + (double)P * B * 4 +
