@@ -86,10 +86,10 @@ __global__ void route_level_kernel(int32_t* __restrict__ node_of, const RT* __re
 // samples go to consecutive positions from off[key], in any order -- every
 // consumer is order-independent, but the evaluator's tiles are cheaper when a
 // tile's samples have one class (eval_slice.cuh).  A block counts the keys of its
-// 4096 samples in shared memory, reserves each key's positions with one atomic,
+// 1024 samples in shared memory, reserves each key's positions with one atomic,
 // then places them.  kSmem = false: too many keys for shared memory, one global
 // atomic per warp and key.
-constexpr int kGroupThreads = 256, kGroupItems = 16;
+constexpr int kGroupThreads = 256, kGroupItems = 4;
 constexpr int kGroupKeys = 8192;  // most keys counted in shared memory
 
 template <bool kSmem, typename KeyOf, typename Put>
@@ -643,8 +643,9 @@ int de_batched(deoct_ctx* ctx, const deoct_dataset* ds, const Compacted& c, uint
   const int P = prm->pop, B = (1 << Dt) - 1, L = 1 << Dt, m2 = 2 * B, K = ds->K, F = ds->F;
   const int W = ds->rank_bytes;
   // per-problem DE state, one block of device memory
-  const size_t per = (size_t)P * m2 * 4 * 2 + (size_t)P * 8 * 2 + 16 + (size_t)P * B * 4 +
-                     (size_t)P * L * K * 4;
+  // (a multiple of 16: every problem's arrays stay aligned whatever P)
+  const size_t per = ((size_t)P * m2 * 4 * 2 + (size_t)P * 8 * 2 + 16 + (size_t)P * B * 4 +
+                      (size_t)P * L * K * 4 + 15) & ~size_t(15);
   unsigned char* blk = nullptr;
   DEOCT_TRY(scratch_get(ctx, SL_MH_POP, per * M + 256 * (size_t)M, (void**)&blk));
   std::vector<DEProb> dp(M);
