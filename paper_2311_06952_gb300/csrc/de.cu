@@ -30,6 +30,11 @@ __device__ __forceinline__ double exact_double(int64_t e) {
   return __longlong_as_double((long long)(((uint64_t)(1086 - lz) << 52) | mant));
 }
 
+// alpha = 0 and alpha >= 0 by its bits (alpha is not NaN): one FP64 comparison costs
+// a warp tens of cycles on this GPU's FP64 pipe, and a step has 4 to 32 warps.
+__device__ __forceinline__ bool is_zero(double x) { return (__double_as_longlong(x) << 1) == 0; }
+__device__ __forceinline__ bool non_negative(double x) { return __double_as_longlong(x) >= 0 || is_zero(x); }
+
 // Fitness order.  With alpha >= 0 every fitness is a non-negative double (not
 // -0), whose bit pattern as a signed 64-bit integer orders exactly like the
 // value, so comparisons need no FP64 arithmetic; a negative alpha compares the
@@ -39,6 +44,14 @@ __device__ __forceinline__ bool fit_le(double x, double y, bool bits) {
 }
 __device__ __forceinline__ bool fit_lt(double x, double y, bool bits) {
   return bits ? __double_as_longlong(x) < __double_as_longlong(y) : x < y;
+}
+
+// Asynchronous copies to shared memory, 16 or 4 bytes.
+__device__ __forceinline__ void cp_async16(void* dst, const void* src) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(dst)), "l"(src) : "memory");
+}
+__device__ __forceinline__ void cp_async4(void* dst, const void* src) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(smem_u32(dst)), "l"(src) : "memory");
 }
 
 __device__ __forceinline__ float clamp_gene(float v, float hi) {
@@ -123,6 +136,13 @@ __global__ void __launch_bounds__(1024) de_init_kernel(const DEArgs a) {
   if (threadIdx.x == 0 && pb.gen) *pb.gen = 1;
 }
 
+// (errors + V) + alpha splits.  A function of its own: inlined beside the integer
+// form for alpha = 0, the compiler computes both and selects, and the FP64
+// operations are most of a small step's selection.
+__device__ __noinline__ double penalised(int64_t ev, double alpha, uint32_t splits) {
+  return __dadd_rn((double)ev, __dmul_rn(alpha, (double)splits));
+}
+
 // The fitness of Section 3.2 of individual r from its class counts,
 //   f = (errors + V) + alpha * splits, errors = n - sum_leaf max_k count,
 //   V = #{leaf : 0 < n_leaf < n_min}, splits = #{t : a_t >= 1} (ahat_t >= 1),
@@ -176,8 +196,8 @@ __device__ double group_fitness(const uint32_t* __restrict__ c, const float* __r
   const int64_t errors = n_valid - (int64_t)correct;
   // alpha = 0 (the default): the fitness is the integer errors + V, and
   // (errors + V) + 0 * splits is that integer exactly
-  if (alpha == 0.0) return exact_double(errors + (int64_t)v);
-  return __dadd_rn((double)(errors + (int64_t)v), __dmul_rn(alpha, (double)splits));
+  if (is_zero(alpha)) return exact_double(errors + (int64_t)v);
+  return penalised(errors + (int64_t)v, alpha, splits);
 }
 
 // Eq. selection of individual r by its group of G lanes: the fitness of its
@@ -267,7 +287,7 @@ __global__ void __launch_bounds__(1024) de_step_kernel(const DEArgs a, int g_arg
   const uint32_t gm = (G == 32 ? 0xFFFFFFFFu : ((1u << G) - 1u)) << ((threadIdx.x & 31) & ~(G - 1));
   const int r0 = threadIdx.x / G, rstep = blockDim.x / G;
 
-  const bool bits = a.alpha >= 0.0;  // fitness order by bit patterns (see fit_lt)
+  const bool bits = non_negative(a.alpha);  // fitness order by bit patterns (see fit_lt)
   if (threadIdx.x == 0) g_s = (flags & DE_GEN_DEVICE) ? *pb.gen : g_arg;
 
   if (flags & (DE_FIRST | DE_SELECT)) {
@@ -300,202 +320,220 @@ __global__ void __launch_bounds__(1024) de_step_kernel(const DEArgs a, int g_arg
 }
 
 // The steady-state step (Eq. selection of generation g - 1's trials, then
-// generation g's trial vectors) when every individual has its own group of G
-// lanes (P G <= 512) and a lane holds at most four consecutive genes (2B <= 4G).
-// The general step waits on global memory once per gene or leaf in turn; here
-// the loads an individual needs that do not wait for the argmin (its class
-// counts, fitness, trial and population genes, and the genes of r1 and r2, whose
-// draws need no memory) are issued together, the argmin reads the fitness from
-// shared memory, and the decode reads the new genes and n_p there too.  The
-// values are those of the general step: integer sums in any order, the same
-// draws, one rounding per float operation, the same selection and argmin.
-constexpr int kFastP = 256, kFastM = 16, kFastC = 16;
+// generation g's trial vectors) of one problem in one CTA with everything on
+// chip.  The general step walks chains of dependent global loads (a gene at a
+// time, the genes of r1, r2 and the best after their draws and the argmin) and
+// every lane of an individual's group computes the Philox blocks it needs, mostly
+// the same ones.  Here the population, the trials, the class counts and n_p are
+// copied to shared memory by asynchronous copies that are all in flight together,
+// each Philox block of an individual is computed once, by one lane, and the rest
+// -- fitness, selection, argmin, mutation, crossover, decoding -- reads shared
+// memory.  What is left is instruction issue on one SM, so the counts come by
+// 16-byte copies and one short loop a leaf (sixteen predicated loads a lane took 6k
+// of 17k cycles), sums are 32-bit, and one warp finds the argmin with warp
+// reductions.  The values are those of the general step: integer sums in any
+// order, the same draws, one rounding per float operation, the same selection and
+// argmin.  Measured on GB300 (a step; before: a register form of this step for
+// depth <= 3, else the general step): P = 64, depth 2 7.9 -> 6.6 us; P = 128, depth 3
+// 10.3 -> 8.4 us; P = 100, depth 4 14.6 -> 8.9 us.  What bounds it is latency: about
+// 700 instructions a warp at ten cycles each, the launch, and four dependent
+// round trips (generation number, copies, stores).
+//
+// Shared memory (step_layout): genes of the population and of the trials [P][m]
+// (the selected rows of the trials are copied over the population's), draws
+// [P][8 nblk], fitness [P], n_p [F], class counts [P][L][K].
+struct StepLayout {
+  int trial, draws, fit, nu, cnt, total;  // byte offsets (the population is at 0)
+};
+__host__ __device__ __forceinline__ StepLayout step_layout(int P, int m, int F, int LK) {
+  const int nblk = (m + 4 + 7) / 8;
+  StepLayout l;
+  l.trial = (P * m * 4 + 15) & ~15;
+  l.draws = 2 * l.trial;
+  l.fit = l.draws + P * nblk * 32;
+  l.nu = (l.fit + P * 8 + 15) & ~15;
+  l.cnt = (l.nu + F * 4 + 15) & ~15;
+  l.total = l.cnt + P * LK * 4;
+  return l;
+}
+constexpr int kStepSmem = 200 * 1024;  // most shared memory of the step
+constexpr int kStepLanes = 3;          // at most 2^3 lanes an individual
+constexpr int kStepP = 256;            // larger populations are split over CTAs (below)
 
-__global__ void __launch_bounds__(512) de_step_fast_kernel(const DEArgs a, int g_arg, int flags,
-                                                          int G) {
-  __shared__ double red_f[32];
-  __shared__ int red_i[32];
+// nw words of global memory to shared memory (dst 16-byte aligned, src of any
+// alignment), asynchronously, by the whole CTA.
+__device__ __forceinline__ void copy_async(uint32_t* dst, const uint32_t* src, int nw) {
+  int done = 0;
+  if ((reinterpret_cast<uintptr_t>(src) & 15) == 0) {
+    done = nw & ~3;
+    for (int e = 4 * threadIdx.x; e < done; e += 4 * blockDim.x) cp_async16(dst + e, src + e);
+  }
+  for (int e = done + threadIdx.x; e < nw; e += blockDim.x) cp_async4(dst + e, src + e);
+}
+
+// Index of the least of fit[0..P) (the lowest of equals), by one warp; in the order
+// of fit_lt.
+__device__ __forceinline__ int warp_argmin(const double* fit, int P, int lane, bool bits) {
+  long long bk = 0x7FFFFFFFFFFFFFFFll;
+  double bf = 0.0;
+  int bi = -1;
+  for (int r = lane; r < P; r += 32) {
+    const double f = fit[r];
+    if (bi < 0 || fit_lt(f, bf, bits)) {
+      bf = f;
+      bi = r;
+    }
+  }
+  if (bits) {  // non-negative doubles: high word, then low word, then index
+    bk = bi < 0 ? bk : __double_as_longlong(bf);
+    const uint32_t hi = (uint32_t)(bk >> 32), lo = (uint32_t)bk;
+    const uint32_t mh = __reduce_min_sync(0xFFFFFFFFu, hi);
+    const uint32_t ml = __reduce_min_sync(0xFFFFFFFFu, hi == mh ? lo : 0xFFFFFFFFu);
+    return (int)__reduce_min_sync(0xFFFFFFFFu, bi >= 0 && hi == mh && lo == ml ? (uint32_t)bi : 0xFFFFFFFFu);
+  }
+  for (int off = 16; off > 0; off >>= 1) {
+    const double of = __shfl_xor_sync(0xFFFFFFFFu, bf, off);
+    const int oi = __shfl_xor_sync(0xFFFFFFFFu, bi, off);
+    if (oi >= 0 && (bi < 0 || of < bf || (!(bf < of) && oi < bi))) {
+      bf = of;
+      bi = oi;
+    }
+  }
+  return bi;
+}
+
+__global__ void __launch_bounds__(1024) de_step_chip_kernel(const DEArgs a, int g_arg, int flags, int lg) {
+  extern __shared__ __align__(16) unsigned char sm[];
   __shared__ int best_s;
-  __shared__ double fit_s[kFastP];
-  __shared__ unsigned char sel_s[kFastP];
-  __shared__ float u_s[kFastP * kFastM];
-  __shared__ uint32_t nu_s[kMaxF];
   const DEProb& pb = prob_of(a);
-  const int P = a.P, B = (1 << a.depth) - 1, m = 2 * B, L = 1 << a.depth, K = pb.K;
-  const int sub = threadIdx.x & (G - 1);
-  const uint32_t gm = (G == 32 ? 0xFFFFFFFFu : ((1u << G) - 1u)) << ((threadIdx.x & 31) & ~(G - 1));
-  const int r = threadIdx.x / G;
+  const int P = a.P, B = (1 << a.depth) - 1, m = 2 * B, L = 1 << a.depth, K = pb.K, F = pb.F, LK = L * K;
+  const int nblk = (m + 4 + 7) / 8, G = 1 << lg;
+  const StepLayout lay = step_layout(P, m, F, LK);
+  float* pop_s = reinterpret_cast<float*>(sm);
+  float* tri_s = reinterpret_cast<float*>(sm + lay.trial);
+  uint32_t* drw_s = reinterpret_cast<uint32_t*>(sm + lay.draws);
+  double* fit_s = reinterpret_cast<double*>(sm + lay.fit);
+  uint32_t* nu_s = reinterpret_cast<uint32_t*>(sm + lay.nu);
+  uint32_t* cnt_s = reinterpret_cast<uint32_t*>(sm + lay.cnt);
+  const int tid = threadIdx.x, NT = blockDim.x;
+  const int sub = tid & (G - 1), r = tid >> lg;
+  const uint32_t gm = (G == 32 ? 0xFFFFFFFFu : ((1u << G) - 1u)) << ((tid & 31) & ~(G - 1));
   const bool act = r < P;  // a whole group is active or not
-  const bool bits = a.alpha >= 0.0;
-  const int per = (m + G - 1) / G;
-  const int q0 = sub * per, q1 = min(m, q0 + per);
-  for (int f = threadIdx.x; f < pb.F; f += blockDim.x) nu_s[f] = pb.n_unique[f];
+  const bool bits = non_negative(a.alpha);
 
-  // ---- this individual's own data (one round of loads) ----------------------
-  // a lane's class counts: leaves sub, sub + G, ..., all K classes of each
-  const int nc = ((L - sub + G - 1) / G) * K;  // at most kFastC (checked at launch)
-  float tr[4], pr[4];
-  uint32_t cv[kFastC];
-  double fr = 0.0;
-  if (act) {
-    fr = pb.fit[r];
-    const float* trg = pb.trial + (int64_t)r * m;
-    const float* pog = pb.pop + (int64_t)r * m;
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const int q = q0 + j;
-      tr[j] = q < q1 ? trg[q] : 0.0f;
-      pr[j] = q < q1 ? pog[q] : 0.0f;
-    }
-    const uint32_t* c = pb.counts + (int64_t)r * L * K;
-    int li = sub, ki = 0;  // leaf and class of the next count loaded
-#pragma unroll
-    for (int e = 0; e < kFastC; ++e) {
-      cv[e] = e < nc ? c[li * K + ki] : 0u;
-      if (++ki == K) {
-        ki = 0;
-        li += G;
-      }
-    }
-  }
-
-  // ---- generation g's draws and the genes of r1 and r2 (no memory needed for
-  // the draws, so they run while the loads above are in flight) --------------
+  // ---- loads, then generation g's draws while they are in flight: block q of
+  // individual i by thread i nblk + q ----------------------------------------------
   const int g = (flags & DE_GEN_DEVICE) ? *pb.gen : g_arg;
+  copy_async(cnt_s, pb.counts, P * LK);
+  copy_async(reinterpret_cast<uint32_t*>(tri_s), reinterpret_cast<const uint32_t*>(pb.trial), P * m);
+  copy_async(reinterpret_cast<uint32_t*>(pop_s), reinterpret_cast<const uint32_t*>(pb.pop), P * m);
+  copy_async(nu_s, pb.n_unique, F);
+  asm volatile("cp.async.commit_group;" ::: "memory");
+  const double fr = act ? pb.fit[r] : 0.0;
   const bool trial = g >= 1 && g <= pb.G;
-  int r1 = 0, r2 = 0, qrand = 0;
-  float M = a.M, rq[4], t1[4], p1[4], t2[4], p2[4];
-  if (act && trial) {
-    const U64x4 blk0 = philox4x64_10((uint64_t)g, (uint64_t)r, 0ull, 0ull, pb.seed, pb.stream_id);
-    const uint32_t x0 = draw_from_block(blk0, 0), x1 = draw_from_block(blk0, 1);
-    const uint32_t x2 = draw_from_block(blk0, 2), x3 = draw_from_block(blk0, 3);
-    r1 = (int)below(x0, (uint32_t)(P - 1));
-    if (r1 >= r) r1 += 1;
-    r2 = (int)below(x1, (uint32_t)(P - 2));
-    const int lo = r < r1 ? r : r1, hi = r < r1 ? r1 : r;
-    if (r2 >= lo) r2 += 1;
-    if (r2 >= hi) r2 += 1;
-    qrand = (int)below(x2, (uint32_t)m);
-    if (a.dither) M = u01(x3);
-    const float* t1g = pb.trial + (int64_t)r1 * m;
-    const float* p1g = pb.pop + (int64_t)r1 * m;
-    const float* t2g = pb.trial + (int64_t)r2 * m;
-    const float* p2g = pb.pop + (int64_t)r2 * m;
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const int q = q0 + j;
-      const bool in = q < q1;
-      t1[j] = in ? t1g[q] : 0.0f;
-      p1[j] = in ? p1g[q] : 0.0f;
-      t2[j] = in ? t2g[q] : 0.0f;
-      p2[j] = in ? p2g[q] : 0.0f;
+  if (trial)
+    for (int e = tid; e < P * nblk; e += NT) {
+      const int i = e / nblk, q = e - i * nblk;
+      const U64x4 b = philox4x64_10((uint64_t)g, (uint64_t)i, (uint64_t)q, 0ull, pb.seed, pb.stream_id);
+      uint4* d = reinterpret_cast<uint4*>(drw_s + e * 8);
+      d[0] = make_uint4((uint32_t)b.x[0], (uint32_t)(b.x[0] >> 32), (uint32_t)b.x[1], (uint32_t)(b.x[1] >> 32));
+      d[1] = make_uint4((uint32_t)b.x[2], (uint32_t)(b.x[2] >> 32), (uint32_t)b.x[3], (uint32_t)(b.x[3] >> 32));
     }
-    // gene q draws s = q + 4 from block s / 8: a lane's four genes touch at most two
-    U64x4 blk = blk0;
-    uint32_t cur = 0;
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const uint32_t s = 4u + (uint32_t)(q0 + j);
-      if (q0 + j < q1 && (s >> 3) != cur) {
-        cur = s >> 3;
-        blk = philox4x64_10((uint64_t)g, (uint64_t)r, (uint64_t)cur, 0ull, pb.seed, pb.stream_id);
-      }
-      rq[j] = u01(draw_from_block(blk, s));
+  asm volatile("cp.async.wait_all;" ::: "memory");
+  __syncthreads();
+
+  // ---- the counts are on chip: zeroed for the next evaluation ---------------------
+  {
+    uint32_t* c = pb.counts;
+    int done = 0;
+    if ((reinterpret_cast<uintptr_t>(c) & 15) == 0) {
+      done = (P * LK) & ~3;
+      for (int e = 4 * tid; trial && e < done; e += 4 * NT) *reinterpret_cast<uint4*>(c + e) = make_uint4(0, 0, 0, 0);
     }
+    for (int e = done + tid; trial && e < P * LK; e += NT) c[e] = 0;
   }
 
-  // ---- the fitness of Section 3.2 from the counts (as group_fitness) ---------
-  double f = 0.0;
+  // ---- the fitness of Section 3.2 of the just-evaluated trial, Eq. selection -------
   if (act) {
-    long long correct = 0;
-    uint32_t v = 0, splits = 0;
-    uint32_t mx = 0;
-    int64_t nl = 0;
-    int kr = 0;  // classes of the current leaf reduced so far
-#pragma unroll
-    for (int e = 0; e < kFastC; ++e) {
-      if (e < nc) {
-        mx = cv[e] > mx ? cv[e] : mx;
-        nl += cv[e];
-        if (++kr == K) {
-          correct += mx;
-          if (nl > 0 && nl < a.n_min) v += 1;
-          mx = 0;
-          nl = 0;
-          kr = 0;
-        }
+    uint32_t correct = 0, vs = 0;  // vs: V below bit 16, splits above
+    const float* tr = tri_s + r * m;
+    for (int l = sub; l < L; l += G) {
+      const uint32_t* c = cnt_s + r * LK + l * K;
+      uint32_t mx = 0, nl = 0;
+      for (int k = 0; k < K; ++k) {
+        const uint32_t x = c[k];
+        mx = x > mx ? x : mx;
+        nl += x;
       }
+      correct += mx;
+      if (nl > 0 && (int64_t)nl < a.n_min) vs += 1;
     }
-    if (a.alpha != 0.0) {
-#pragma unroll
-      for (int j = 0; j < 4; ++j)
-        if (q0 + j < q1 && q0 + j < B) splits += tr[j] >= 1.0f ? 1u : 0u;
-    }
+    if (!is_zero(a.alpha))
+      for (int t = sub; t < B; t += G) vs += tr[t] >= 1.0f ? 0x10000u : 0u;
     for (int o = G >> 1; o > 0; o >>= 1) {
       correct += __shfl_xor_sync(gm, correct, o);
-      v += __shfl_xor_sync(gm, v, o);
-      splits += __shfl_xor_sync(gm, splits, o);
+      vs += __shfl_xor_sync(gm, vs, o);
     }
-    const int64_t errors = pb.n_valid - (int64_t)correct;
-    f = (a.alpha == 0.0) ? exact_double(errors + (int64_t)v)
-                         : __dadd_rn((double)(errors + (int64_t)v), __dmul_rn(a.alpha, (double)splits));
-  }
-
-  // ---- Eq. selection, then the argmin over shared memory --------------------
-  bool take = false;
-  if (act) {
-    __syncwarp(gm);  // every lane has read fit[r] before it is rewritten
-    take = fit_le(f, fr, bits);  // ties go to the trial
-    if (sub == 0) pb.fit_trial[r] = f;
+    const int64_t ev = pb.n_valid - (int64_t)correct + (int64_t)(vs & 0xFFFFu);  // errors + V
+    const double f = is_zero(a.alpha) ? exact_double(ev) : penalised(ev, a.alpha, vs >> 16);
+    const bool take = fit_le(f, fr, bits);  // ties go to the trial
     if (take) {
-      float* dst = pb.pop + (int64_t)r * m;
-#pragma unroll
-      for (int j = 0; j < 4; ++j)
-        if (q0 + j < q1) dst[q0 + j] = tr[j];
-      if (sub == 0) pb.fit[r] = f;
+      float *po = pop_s + r * m, *dst = pb.pop + (int64_t)r * m;
+      for (int q = sub; q < m; q += G) {
+        const float x = tr[q];
+        po[q] = x;
+        dst[q] = x;
+      }
     }
     if (sub == 0) {
+      pb.fit_trial[r] = f;
+      if (take) pb.fit[r] = f;
       fit_s[r] = take ? f : fr;
-      sel_s[r] = take ? 1 : 0;
     }
   }
   __syncthreads();
-  block_argmin(fit_s, P, &best_s, red_f, red_i, bits);
-  if (threadIdx.x == 0) *pb.best = best_s;
-  if (!trial) return;  // device-driven replay past the last generation
-
-  // ---- generation g's trial vectors from the new population, decoded --------
-  if (act) {
-    const float ub_a = (float)(pb.F + 1);
-    const float hi_a = below_bound(ub_a), hi_b = below_bound(1.0f);
-    const float* sbg = pb.pop + (int64_t)best_s * m;  // the new population: copies are done
-    const bool sel1 = sel_s[r1] != 0, sel2 = sel_s[r2] != 0;
-    float* u = pb.trial + (int64_t)r * m;
-    float* us = u_s + r * m;
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const int q = q0 + j;
-      if (q < q1) {
-        const float s1 = sel1 ? t1[j] : p1[j], s2 = sel2 ? t2[j] : p2[j];
-        const float sr = take ? tr[j] : pr[j];
-        const float v = __fadd_rn(sbg[q], __fmul_rn(M, __fsub_rn(s1, s2)));
-        const float vc = clamp_gene(v, q < B ? hi_a : hi_b);
-        const float uq = (rq[j] <= a.CR || q == qrand) ? vc : sr;
-        u[q] = uq;
-        us[q] = uq;
-      }
+  if (tid < 32) {
+    const int b = warp_argmin(fit_s, P, tid, bits);
+    if (tid == 0) {
+      best_s = b;
+      *pb.best = b;
     }
-    __syncwarp(gm);  // the group's genes are in shared memory before they are decoded
+  }
+  if (!trial) return;  // device-driven replay past the last generation (uniform)
+  __syncthreads();
+
+  // ---- generation g's trial vectors from the new population, decoded --------------
+  if (act) {
+    const float hi_a = below_bound((float)(F + 1)), hi_b = below_bound(1.0f);
+    const uint32_t* dr = drw_s + r * nblk * 8;
+    int r1 = (int)below(dr[0], (uint32_t)(P - 1));
+    if (r1 >= r) r1 += 1;
+    int r2 = (int)below(dr[1], (uint32_t)(P - 2));
+    const int lo = r < r1 ? r : r1, hi = r < r1 ? r1 : r;
+    if (r2 >= lo) r2 += 1;
+    if (r2 >= hi) r2 += 1;
+    const int qrand = (int)below(dr[2], (uint32_t)m);
+    const float M = a.dither ? u01(dr[3]) : a.M;
+    const float *sb = pop_s + best_s * m, *s1 = pop_s + r1 * m, *s2 = pop_s + r2 * m, *sr = pop_s + r * m;
+    float* u = pb.trial + (int64_t)r * m;
+    // u01(x) <= CR with u01(x) = (x >> 8) 2^-24, in integers (CR 2^24 is exact)
+    const uint32_t cr24 = (uint32_t)floorf(__fmul_rn(a.CR, 16777216.0f));
+    auto gene = [&](int q, float top) {
+      const float x = __fadd_rn(sb[q], __fmul_rn(M, __fsub_rn(s1[q], s2[q])));
+      const float xc = clamp_gene(x, top);
+      const float uq = ((dr[4 + q] >> 8) <= cr24 || q == qrand) ? xc : sr[q];
+      u[q] = uq;
+      return uq;
+    };
     for (int t = sub; t < B; t += G) {
+      const float ah = gene(t, hi_a), bh = gene(B + t, hi_b);
       int av;
       uint32_t th;
-      decode_gene_pair(us[t], us[B + t], pb.F, nu_s, &av, &th);
+      decode_gene_pair(ah, bh, F, nu_s, &av, &th);
       pb.nodes[(int64_t)r * B + t] = pack_node(av, th);
     }
   }
-  const int64_t total = (int64_t)P * L * K;  // every count was read before the barrier
-  for (int64_t e = threadIdx.x; e < total; e += blockDim.x) pb.counts[e] = 0;
-  if (threadIdx.x == 0 && (flags & DE_GEN_DEVICE)) *pb.gen = g + 1;
+  if (tid == 0 && (flags & DE_GEN_DEVICE)) *pb.gen = g + 1;
 }
 
 // The steady-state step of one problem with a large population, split over CTAs
@@ -518,7 +556,7 @@ __global__ void __launch_bounds__(kDeWideR * kDeWideG) de_select_wide_kernel(con
   const uint32_t gm = ((1u << G) - 1u) << ((threadIdx.x & 31) & ~(G - 1));
   const int r0 = blockIdx.x * kDeWideR, nr = min(kDeWideR, P - r0);
   const int r = r0 + (int)threadIdx.x / G;
-  const bool bits = a.alpha >= 0.0;
+  const bool bits = non_negative(a.alpha);
   if (r < P) select_individual(a, pb, r, B, L, K, sub, G, gm, bits);  // whole groups only
   __syncthreads();
   block_argmin(pb.fit + r0, nr, &best_s, red_f, red_i, bits);
@@ -542,7 +580,7 @@ __global__ void __launch_bounds__(kDeWideR * kDeWideG) de_trial_wide_kernel(cons
   const uint32_t gm = ((1u << G) - 1u) << ((threadIdx.x & 31) & ~(G - 1));
   const int r0 = blockIdx.x * kDeWideR, nr = min(kDeWideR, P - r0);
   const int r = r0 + (int)threadIdx.x / G;
-  block_argmin(a.part_f, nblk, &best_s, red_f, red_i, a.alpha >= 0.0);
+  block_argmin(a.part_f, nblk, &best_s, red_f, red_i, non_negative(a.alpha));
   const int best = a.part_i[best_s];
   const int g = *a.part_g;
   const bool trial = g >= 1 && g <= pb.G;  // false: device-driven replay past the last generation
@@ -620,16 +658,17 @@ int de_launch_step(deoct_ctx* ctx, const DEArgs& a, int g, int flags, cudaStream
   if (nprob <= 0) return DEOCT_OK;
   const int lanes = lanes_for(a.P);
   const int m = 2 * ((1 << a.depth) - 1);
-  const int L = 1 << a.depth;
-  if ((flags & DE_SELECT) && (flags & DE_TRIAL) && !(flags & DE_FIRST) && a.P * lanes <= 512 &&
-      a.P <= kFastP && m <= 4 * lanes && m <= kFastM && a.Kmax > 0 &&
-      ((L + lanes - 1) / lanes) * a.Kmax <= kFastC) {
-    de_step_fast_kernel<<<nprob, block_for(a.P * lanes), 0, s>>>(a, g, flags, lanes);
+  const bool steady = (flags & DE_SELECT) && (flags & DE_TRIAL) && !(flags & DE_FIRST);
+  const size_t smem = a.Kmax > 0 ? (size_t)step_layout(a.P, m, kMaxF, (1 << a.depth) * a.Kmax).total : kStepSmem + 1;
+  if (steady && a.P <= kStepP && smem <= (size_t)kStepSmem) {
+    int lg = 0;  // lanes an individual (log2)
+    while (lg < kStepLanes && (2 << lg) <= (1 << a.depth) && (a.P << lg) * 2 <= 1024) ++lg;
+    DEOCT_TRY(set_max_dynamic_smem(ctx, de_step_chip_kernel));
+    de_step_chip_kernel<<<nprob, block_for(a.P << lg), smem, s>>>(a, g, flags, lg);
     count_launch(ctx);
-    return check_launch("de_step_fast_kernel");
+    return check_launch("de_step_chip_kernel");
   }
-  if ((flags & DE_SELECT) && (flags & DE_TRIAL) && !(flags & DE_FIRST) && !a.probs && a.part_f &&
-      a.P > kFastP && a.P <= kMaxPop) {
+  if (steady && !a.probs && a.part_f && a.P > kStepP && a.P <= kMaxPop) {
     const int nblk = (a.P + kDeWideR - 1) / kDeWideR;
     de_select_wide_kernel<<<nblk, kDeWideR * kDeWideG, 0, s>>>(a, g, flags);
     count_launch(ctx);
