@@ -1381,7 +1381,7 @@ size_t fit_scratch_bound(const deoct_ctx* ctx, int64_t n, int F, int K, int W, c
   for (int sl : {SL_ENC_K0, SL_ENC_K1, SL_ENC_V0, SL_ENC_V1}) need(sl, 4.0 * nF);
   need(SL_ENC_TILE, 4.0 * F * tiles);
   need(SL_ENC_HIST, 4.0 * F * 256 * tiles);
-  need(SL_ENC_TOT, 4.0 * F * 256);
+  need(SL_ENC_TOT, 4.0 * F * 1024 + 64);
   // moving horizon: level state and compacted segments
   const int64_t npad = round_up(n + (int64_t)kSegAlign * nn, 64);
   const int64_t ptiles = (npad + 2047) / 2048;
