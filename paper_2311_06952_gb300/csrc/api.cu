@@ -199,12 +199,12 @@ static int slice_planes_of_fit(deoct_ctx* ctx, const deoct_dataset* ds, const in
   return slc::slice_planes(ctx, ds->rank_bytes, *plan, nullptr, 1, tiles, s);
 }
 
-// One evaluation on its own: trees from which the bit-sliced evaluator, which then
-// transposes every tile's ranks itself, is the faster one (GB300: 100 to 128 trees
-// 150 us against 145 at n = 1e6, F = 30, depth 3, 49 against 45 at n = 2e5, K = 10;
-// 256 trees 500 us against 790 at n = 2e6, depth 5; 1024 trees 4.5 ms against 10.2
-// at n = 1e7, depth 4).
-constexpr int kSliceOnce = 192;
+// One evaluation on its own: whether the bit-sliced evaluator, which then transposes
+// every tile's ranks itself, is the faster one (GB300: 100 to 128 trees 150 us against
+// 145 at n = 1e6, F = 30, depth 3, 49 against 45 at n = 2e5, K = 10; 256 trees 39
+// against 35 us at n = 1e5, F = 20, depth 3, 500 against 790 at n = 2e6, depth 5; 1024
+// trees 4.5 ms against 10.2 at n = 1e7, depth 4).
+static bool slice_once(int64_t n_sub, int P) { return P >= 192 && n_sub * P >= (int64_t(1) << 27); }
 
 // Bound of an encoded set's ranks that needs no look at the device: its size, and
 // the rank width.  (Where a set breaks it the evaluator still counts right, slowly.)
@@ -227,7 +227,7 @@ static int eval_single(deoct_ctx* ctx, const deoct_dataset* ds, const int32_t* i
   if (n_sub == 0) return DEOCT_OK;
   EvalPlan sp;
   slc::SliceShape sh;
-  if (P >= kSliceOnce && slice_plan(ctx, ds, idx, n_sub, P, depth, width_bound(ds), &sp, &sh)) {
+  if (slice_once(n_sub, P) && slice_plan(ctx, ds, idx, n_sub, P, depth, width_bound(ds), &sp, &sh)) {
     sp.single.nodes = nodes;
     sp.single.counts = counts;
     return slc::slice_launch(ctx, depth, sp, sh, s);
@@ -251,7 +251,7 @@ static int eval_single_fused(deoct_ctx* ctx, const deoct_dataset* ds, const int3
   if (grows) DEOCT_CUDA_TRY(cudaMemsetAsync(base, 0, ctx->scratch[SL_EVAL_ACC].bytes, s));
   EvalPlan sp;
   slc::SliceShape sh;
-  if (P >= kSliceOnce && slice_plan(ctx, ds, idx, n_sub, P, depth, width_bound(ds), &sp, &sh)) {
+  if (slice_once(n_sub, P) && slice_plan(ctx, ds, idx, n_sub, P, depth, width_bound(ds), &sp, &sh)) {
     sp.single.a16 = a;
     sp.single.th32 = theta;
     sp.single.counts = base + 4;

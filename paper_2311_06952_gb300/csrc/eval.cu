@@ -72,8 +72,13 @@ __global__ void __launch_bounds__(1024, 1) eval_kernel(const __grid_constant__ E
       __syncthreads();
       jv = nv;
       cur_job = nv.job;
-      setup_job<D, Q, MODE == 0>(jv, nodes_s, cnt_s, tile_sa, S, W, a.status, lane, blockDim.x, cst,
-                                 &K, &LK);
+      if (MODE == 0) {
+        setup_job<D, Q, true>(jv, nodes_s, cnt_s, tile_sa, S, W, a.status, lane, blockDim.x, cst, &K, &LK);
+      } else {
+        K = jv.p->K;
+        LK = L * K;
+        setup_packed<D>(jv, reinterpret_cast<uint32_t*>(nodes_s), cnt_s, LK, a.status, blockDim.x);
+      }
     }
     jv.tile = nv.tile;  // the tile changes every iteration, the job only sometimes
     const EvalProb& P = *jv.p;
@@ -196,23 +201,46 @@ __global__ void __launch_bounds__(1024, 1) eval_kernel(const __grid_constant__ E
       route_group<W, D, Q, false>(jv.ntrees, npair, 0u, nodes_s, nodes_sa, aux_sa, cst, cnt_s, LK,
                                   lane, warp, nw);
     } else {
-      // shared-atomic mode (many bins): all warps work on one tree at a time,
-      // splitting its chunks, and add into the job's shared counts
-      for (int i = 0; i < jv.ntrees; ++i) {
-        const uint32_t tnb = nodes_sa + (uint32_t)(i * B - 1) * 8u;
+      // shared-atomic mode (many bins): a warp walks a tree over the tile two chunks
+      // at a time (or, with fewer trees than half the warps, the warps split each
+      // tree's chunks) and adds into the job's shared counts.  Nodes are one packed
+      // word (half the bank conflicts and memory of {address, theta} pairs); the root
+      // and level 1 are held in registers.  Issue bounds it (62% of the slots, about
+      // 100 instructions per 32 samples and tree at depth 8).  GB300, one evaluation
+      // (before: all warps on one tree at a time, and the last CTA's errors by one thread
+      // a tree): n = 1e6, F = 28, 100 trees of depth 8 580 -> 400 us; n = 3e5, 300 trees of
+      // depth 7 500 -> 286; n = 2e6, K = 29, 32 trees of depth 8 1337 -> 529; n = 5000, 100
+      // trees of depth 8 254 -> 39.
+      const uint32_t* nodes32 = reinterpret_cast<const uint32_t*>(nodes_s);
+      const uint32_t SW = (uint32_t)(S * W);
+      const bool own = 2 * jv.ntrees > nw;
+      for (int i = own ? warp : 0; i < jv.ntrees; i += own ? nw : 1) {
+        const uint32_t tnb = nodes_sa + (uint32_t)(i * B - 1) * 4u;
+        const uint32_t n1 = nodes32[i * B], n2 = D >= 2 ? nodes32[i * B + 1] : 0u, n3 = D >= 2 ? nodes32[i * B + 2] : 0u;
         uint32_t* ci = cnt_s + i * LK;
-        for (int c = warp; c < nch; c += nw) {
-          const uint32_t j = (uint32_t)(c * 32 + lane);
-          const uint32_t jo = tile_offset<W>(j);
-          uint32_t t = 1;
-#pragma unroll
-          for (int d = 0; d < D; ++d) {
-            const uint2 nd = lds_node(tnb + 8u * t);
-            uint32_t rv = lds_rank<W>(nd.x + jo);
-            t = 2 * t + (rv >= nd.y ? 1u : 0u);
-          }
-          const uint32_t y = lab_s[j];
+        auto right = [&](uint32_t nd, uint32_t jo) {  // 1: the sample at jo goes right at node nd
+          return lds_rank<W>((nd >> 24) * SW + jo) >= (nd & kThetaMask) ? 1u : 0u;
+        };
+        auto count = [&](uint32_t t, uint32_t y) {
           if (y < (uint32_t)K) atomicAdd(ci + (t - L) * K + y, 1u);
+        };
+        const int c0 = own ? 0 : warp, cs = own ? 1 : nw;
+        for (int p = c0; p < npair; p += cs) {  // chunks 2 p and 2 p + 1 (both are staged)
+          const uint32_t j = (uint32_t)(p * 64 + lane);
+          const uint32_t ja = tile_sa + tile_offset<W>(j), jb = tile_sa + tile_offset<W>(j + 32u);
+          uint32_t ta = 2u + right(n1, ja), tb = 2u + right(n1, jb);
+          if (D >= 2) {
+            ta = 2u * ta + right(ta == 3u ? n3 : n2, ja);
+            tb = 2u * tb + right(tb == 3u ? n3 : n2, jb);
+          }
+#pragma unroll
+          for (int d = 2; d < D; ++d) {
+            const uint32_t na = lds_u32(tnb + 4u * ta), nb = lds_u32(tnb + 4u * tb);
+            ta = 2u * ta + right(na, ja);
+            tb = 2u * tb + right(nb, jb);
+          }
+          count(ta, lab_s[j]);
+          count(tb, lab_s[j + 32]);
         }
       }
     }
@@ -436,16 +464,29 @@ EvalConfig eval_choose_config(deoct_ctx* ctx, int W, int D, int F, int K, int P,
       }
     }
   } else {
-    // shared-atomic mode: the 16 warps split the chunks of one tree at a time, so
-    // the tile keeps at least 16 chunks (512 samples); the tile shrinks to that
-    // before the group does, since every tree of a group reuses the staged tile
-    // (wide uint32 data would otherwise end at one tree per group and restage
-    // each tile once per tree), and the job's counts ([TG][2^D K]) set TG
+    // shared-atomic mode: a warp takes a tree, so groups are multiples of the 16
+    // warps where the population and shared memory allow, on the largest tile of
+    // 1024 or 512 samples that leaves room for them beside a second CTA (wide uint32
+    // data would otherwise end at one tree per group and restage each tile once per
+    // tree); fewer trees split a tree's chunks over the warps
     c.S = 1024;
     c.warps = 16;
-    c.TG = std::min(P, 256);
-    while (eval_smem(mode, W, D, c.S, c.TG, F, K, c.warps) > two_per_sm && c.S > 512) c.S /= 2;
-    while (eval_smem(mode, W, D, c.S, c.TG, F, K, c.warps) > two_per_sm && c.TG > 1) c.TG /= 2;
+    auto most = [&](int S) {  // trees a group may have
+      int t = std::min(P, 256);
+      while (t > 0 && eval_smem(mode, W, D, S, t, F, K, c.warps) > two_per_sm) --t;
+      return t;
+    };
+    int tg = most(1024);
+    if (tg < std::min(P, 16)) {
+      c.S = 512;
+      tg = most(512);
+    }
+    if (tg >= 16) {
+      tg = tg / 16 * 16;
+      const int groups = (P + tg - 1) / tg;
+      tg = std::min(tg, ((P + groups - 1) / groups + 15) / 16 * 16);
+    }
+    c.TG = std::max(1, std::min(tg, P));
     while (eval_smem(mode, W, D, c.S, c.TG, F, K, c.warps) > (size_t)limit && c.S > 128) c.S /= 2;
     while (work(c.S, c.TG) < 2 * (int64_t)ctx->num_sms && c.TG > 1) c.TG /= 2;
   }

@@ -104,3 +104,31 @@ def test_fit_planes(c, n, K, depth, subset):
         np.testing.assert_array_equal(pop.cpu().numpy().view(np.uint32), ref["pop"].view(np.uint32))
         assert f == ref["fit"][ref["best"]]
         ctx.close()
+
+
+@pytest.mark.parametrize("n,P,W,depth,K", [(32_768, 4096, 2, 3, 2), (32_769, 4099, 4, 2, 3), (33_791, 4096, 2, 4, 5),
+                                           (700_001, 195, 4, 1, 4)])
+def test_one_large_evaluation(c, n, P, W, depth, K):
+    """Single evaluations large enough for the kernel to transpose the ranks itself."""
+    rng = _rng(n)
+    X = (np.floor(rng.random((n, 6)) * 9000) / 9000).astype(np.float32)
+    y = rng.integers(0, K, n).astype(np.uint8)
+    ranks, nu = oracle.encode(X)
+    a, th = datagen.random_population(nu, P, depth, rng, allow_nosplit=True)
+    _check(c, gpu_dataset(c, X, y, K, W), ranks, y, K, a, th, depth)
+
+
+@pytest.mark.parametrize("W,top", [(2, 65_535), (2, (1 << 24) - 1), (4, (1 << 24) - 1)])
+def test_large_evaluation_past_the_set(c, W, top):
+    """The same on a view of a larger encoded set with thresholds past it: the general path."""
+    from paper_2311_06952_gb300 import deoct
+    rng = _rng(W + top + 1)
+    n, F, K, P, depth, part = 30_000, 6, 3, 90_000, 2, 1501
+    X = rng.random((n, F)).astype(np.float32)
+    y = rng.integers(0, K, n).astype(np.uint8)
+    ranks, nu = oracle.encode(X)
+    a, th = datagen.random_population(nu, P, depth, rng, allow_nosplit=True)
+    th[::7] = np.where(a[::7] > 0, top, 0)
+    full = gpu_dataset(c, X, y, K, W)
+    view = deoct.DeviceDataset(full.ranks, W, full.n_unique, full.labels, part, F, K)
+    _check(c, view, ranks[:, :part], y[:part], K, a, th, depth)
