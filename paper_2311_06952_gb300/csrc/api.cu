@@ -356,56 +356,73 @@ int run_deoct(deoct_ctx* ctx, const deoct_dataset* ds, const int32_t* idx, int64
     if (p->gens >= 1) DEOCT_TRY(slice_planes_of_fit(ctx, ds, idx, n_sub, &sp, s));
     sh.raw = sp.single.planes == nullptr;
   }
-  auto evaluate = [&](cudaStream_t st) {
-    return sliced ? slc::slice_launch(ctx, p->depth, sp, sh, st)
+  auto evaluate = [&](cudaStream_t st, bool chained) {
+    return sliced ? slc::slice_launch(ctx, p->depth, sp, sh, st, chained)
                   : eval_ballot(ctx, ds, idx, n_sub, b.nodes, b.counts, p->pop, p->depth, st);
   };
-  DEOCT_TRY(evaluate(s));
+  DEOCT_TRY(evaluate(s, false));
   // The generation number lives on the device (set to 1 by the init kernel and
-  // advanced by every trial step), so every generation is the same pair of
-  // launches: captured once as a CUDA graph and replayed G times.  With
-  // per-launch timing on, the launches are issued directly so that each
-  // evaluator launch gets its own events.
+  // advanced by every trial step), so every generation is the same launches: captured
+  // as CUDA graphs and replayed.  With per-launch timing on, the launches are issued
+  // directly so that each evaluator launch gets its own events.
   DEOCT_TRY(de_launch_step(ctx, a, 0, DE_FIRST | DE_GEN_DEVICE | (p->gens >= 1 ? DE_TRIAL : 0), s));
   if (p->gens < 1) return DEOCT_OK;
   if (ctx->timing || p->gens < 3) {
     for (int g = 1; g <= p->gens; ++g) {
-      DEOCT_TRY(evaluate(s));
+      DEOCT_TRY(evaluate(s, false));
       DEOCT_TRY(de_launch_step(ctx, a, 0, DE_SELECT | DE_TRIAL | DE_GEN_DEVICE, s));
     }
     return DEOCT_OK;
   }
+  return replay_generations(
+      ctx, p->gens,
+      [&](cudaStream_t st) {
+        DEOCT_TRY(evaluate(st, true));
+        return de_launch_step(ctx, a, 0, DE_SELECT | DE_TRIAL | DE_GEN_DEVICE | DE_CHAINED, st);
+      },
+      s);
+}
+
+// Generations captured in one graph: a kernel of a graph may start before the one
+// ahead of it has ended (launch_chained), across graph launches it may not.
+constexpr int kGensPerGraph = 8;
+
+int replay_generations(deoct_ctx* ctx, int G, const std::function<int(cudaStream_t)>& record, cudaStream_t s) {
   if (!ctx->cap_stream)
     DEOCT_CUDA_TRY(cudaStreamCreateWithFlags(&ctx->cap_stream, cudaStreamNonBlocking));
-  const uint64_t l0 = ctx->launches, e0 = ctx->eval_launches;
-  cudaGraph_t graph = nullptr;
-  cudaGraphExec_t exec = nullptr;
-  DEOCT_CUDA_TRY(cudaStreamBeginCapture(ctx->cap_stream, cudaStreamCaptureModeThreadLocal));
-  int rc = evaluate(ctx->cap_stream);
-  if (rc == DEOCT_OK) rc = de_launch_step(ctx, a, 0, DE_SELECT | DE_TRIAL | DE_GEN_DEVICE, ctx->cap_stream);
-  cudaError_t ce = cudaStreamEndCapture(ctx->cap_stream, &graph);
-  const uint64_t per_launch = ctx->launches - l0, per_eval = ctx->eval_launches - e0;
-  ctx->launches = l0;
-  ctx->eval_launches = e0;
-  if (rc != DEOCT_OK) {
-    if (graph) cudaGraphDestroy(graph);
-    return rc;
-  }
-  if (ce != cudaSuccess) return set_error(DEOCT_ERR_CUDA, "graph capture failed: %s", cudaGetErrorString(ce));
-  ce = cudaGraphInstantiate(&exec, graph, 0);
-  if (ce != cudaSuccess) {
+  for (const int gens : {std::min(G, kGensPerGraph), G % std::min(G, kGensPerGraph)}) {
+    if (gens == 0) break;
+    const int replays = gens == std::min(G, kGensPerGraph) ? G / gens : 1;
+    const uint64_t l0 = ctx->launches, e0 = ctx->eval_launches;
+    cudaGraph_t graph = nullptr;
+    cudaGraphExec_t exec = nullptr;
+    DEOCT_CUDA_TRY(cudaStreamBeginCapture(ctx->cap_stream, cudaStreamCaptureModeThreadLocal));
+    int rc = DEOCT_OK;
+    for (int i = 0; i < gens && rc == DEOCT_OK; ++i) rc = record(ctx->cap_stream);
+    cudaError_t ce = cudaStreamEndCapture(ctx->cap_stream, &graph);
+    const uint64_t per_launch = ctx->launches - l0, per_eval = ctx->eval_launches - e0;
+    ctx->launches = l0;
+    ctx->eval_launches = e0;
+    if (rc != DEOCT_OK) {
+      if (graph) cudaGraphDestroy(graph);
+      return rc;
+    }
+    if (ce != cudaSuccess) return set_error(DEOCT_ERR_CUDA, "graph capture failed: %s", cudaGetErrorString(ce));
+    ce = cudaGraphInstantiate(&exec, graph, 0);
+    if (ce != cudaSuccess) {
+      cudaGraphDestroy(graph);
+      return set_error(DEOCT_ERR_CUDA, "graph instantiate failed: %s", cudaGetErrorString(ce));
+    }
+    for (int r = 0; r < replays && ce == cudaSuccess; ++r) {
+      ce = cudaGraphLaunch(exec, s);
+      ctx->launches += per_launch;
+      ctx->eval_launches += per_eval;
+    }
+    // the graph may be destroyed once its launches are queued
+    cudaGraphExecDestroy(exec);
     cudaGraphDestroy(graph);
-    return set_error(DEOCT_ERR_CUDA, "graph instantiate failed: %s", cudaGetErrorString(ce));
+    if (ce != cudaSuccess) return set_error(DEOCT_ERR_CUDA, "graph launch failed: %s", cudaGetErrorString(ce));
   }
-  for (int g = 1; g <= p->gens && ce == cudaSuccess; ++g) {
-    ce = cudaGraphLaunch(exec, s);
-    ctx->launches += per_launch;
-    ctx->eval_launches += per_eval;
-  }
-  // the graph may be destroyed once its launches are queued
-  cudaGraphExecDestroy(exec);
-  cudaGraphDestroy(graph);
-  if (ce != cudaSuccess) return set_error(DEOCT_ERR_CUDA, "graph launch failed: %s", cudaGetErrorString(ce));
   return DEOCT_OK;
 }
 

@@ -261,7 +261,8 @@ int rebuild(deoct_engine* e, const EngineGroupKey& k, Group& g) {
   DEOCT_CUDA_TRY(cudaStreamBeginCapture(c->cap_stream, cudaStreamCaptureModeThreadLocal));
   int rc = sliced ? slc::slice_launch(c, k.Dt, plan, sh, c->cap_stream)
                   : eval_launch(c, k.W, k.Dt, plan, cfg, c->cap_stream);
-  if (rc == DEOCT_OK) rc = de_launch_step(c, a, 0, DE_SELECT | DE_TRIAL | DE_GEN_DEVICE, c->cap_stream);
+  if (rc == DEOCT_OK)
+    rc = de_launch_step(c, a, 0, DE_SELECT | DE_TRIAL | DE_GEN_DEVICE | DE_CHAINED, c->cap_stream);
   cudaError_t ce = cudaStreamEndCapture(c->cap_stream, &graph);
   g.per_replay_launches = c->launches - l0;
   g.per_replay_evals = c->eval_launches - v0;

@@ -56,6 +56,7 @@ struct SliceArgs {
   int rows;         // thermometer rows in shared memory
   int ymask_off, rec_off, acc_off, smem_bytes;
   int rec_bytes;    // node records of one warp
+  bool chained;     // launched with programmatic dependence on the kernel before
 };
 
 // Digit counts the kernel is built for, ascending.
@@ -478,7 +479,7 @@ struct Trees {
   __device__ __forceinline__ explicit Trees(const EvalProb& P) : nodes(P.nodes), a16(P.a16), th32(P.th32), F(P.F) {}
 };
 __device__ __forceinline__ uint32_t fetch_node(const Trees& T, int64_t e, int* status) {
-  if (T.a16 == nullptr) return __ldg(T.nodes + e);
+  if (T.a16 == nullptr) return __ldcg(T.nodes + e);  // from L2: a chained launch may share an SM with its writers
   int av = T.a16[e];
   const uint32_t tv = T.th32[e];
   if (av > T.F || (av > 0 && tv > kThetaMask)) {
@@ -655,13 +656,17 @@ __device__ __forceinline__ void route_tile(const Digits* dg, const EvalProb& P, 
   int i = warp * kTreesPerWarp + q;
   if (warp * kTreesPerWarp >= ntrees) return;
   uint32_t next = subtree_node(i, 0);
+  auto prefix_node = [&](int i) {  // the lane's node above the subtrees of local tree i
+    const int ic = i < ntrees ? i : ntrees - 1;
+    return l8 < S::kSubs - 1 ? fetch_node(T, (int64_t)(tree0 + ic) * B + l8, status) : 0u;
+  };
+  static_assert(S::kSubs - 1 <= 8, "a lane per prefix node");
+  uint32_t pnext = S::kPrefix > 0 ? prefix_node(i) : 0u;
   for (; i - q < ntrees; i += step) {
     if constexpr (S::kPrefix > 0) {
-      const int ic = i < ntrees ? i : ntrees - 1;
       __syncwarp();
-      for (int t = l8; t < S::kSubs - 1; t += 8)
-        put_record<ND>(rd, fetch_node(T, (int64_t)(tree0 + ic) * B + t, status), tmax, therm_sa,
-                       prec + t * RB);
+      if (l8 < S::kSubs - 1) put_record<ND>(rd, pnext, tmax, therm_sa, prec + l8 * RB);
+      pnext = prefix_node(i + step);
     }
     uint4 G[S::kPrefix > 0 ? S::kPrefix : 1];
     uint32_t* acc = accb + (i < ntrees ? i : 0) * accw;
@@ -769,6 +774,11 @@ __global__ void __launch_bounds__(kWarps * 32, 1) eval_slice_kernel(const __grid
   const int64_t T = a.total_tiles;
   const int64_t t0 = (int64_t)blockIdx.x * T / gridDim.x;
   const int64_t t1 = (int64_t)(blockIdx.x + 1) * T / gridDim.x;
+  // Chained launches (a fit's generations): the trees and the zeroed counts are the
+  // previous step's; planes, jobs and problems are older, so the first tile is built
+  // before the wait.
+  bool waited = RAW;
+  if (RAW) chain_wait();
   bool fit = true;  // the job's thetas fit the rows (uniform)
   int cur_job = -1, held = 0;  // held: tiles in the 16-bit counts
   evk::JobView jv;
@@ -825,6 +835,10 @@ __global__ void __launch_bounds__(kWarps * 32, 1) eval_slice_kernel(const __grid
       __syncthreads();  // a digit's task reads planes that other warps left
     }
     build_tile<ND, RAW>(&dg, blk, P.F, P.K, P.nb, therm_sa, ymask_sa, &s_classes, lane, warp);
+    if (!waited) {
+      chain_wait();
+      waited = true;
+    }
     // the CTA's next tile on its way to L2 while this one is routed
     if (gt + 1 < t1 && jv.tile + 1 < jv.ntiles) {
       if constexpr (!RAW) {
@@ -844,6 +858,7 @@ __global__ void __launch_bounds__(kWarps * 32, 1) eval_slice_kernel(const __grid
       }
     }
     __syncthreads();
+    if (gt + 1 == t1) chain_release();  // the step that follows may be set up now
     route_tile<D, ND>(&dg, P, jv.tree0, jv.ntrees, accw, therm_sa, ymask_sa, rec, acc, s_classes, a.status,
                       lane, warp);
     ++held;
@@ -859,7 +874,7 @@ template <int D, int ND>
 int launch_slice_t(deoct_ctx* ctx, const SliceArgs& sa, bool raw, int grid, cudaStream_t s) {
   auto* kern = raw ? eval_slice_kernel<D, ND, true> : eval_slice_kernel<D, ND, false>;
   DEOCT_TRY(set_max_dynamic_smem(ctx, kern));
-  kern<<<grid, kWarps * 32, sa.smem_bytes, s>>>(sa);
+  DEOCT_CUDA_TRY(launch_chained(sa.chained, kern, grid, kWarps * 32, (size_t)sa.smem_bytes, s, sa));
   count_launch(ctx);
   return check_launch("eval_slice_kernel");
 }

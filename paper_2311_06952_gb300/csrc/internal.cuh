@@ -1,6 +1,8 @@
 // internal.cuh -- declarations shared by the translation units of libdeoct.
 #pragma once
 
+#include <functional>
+
 #include "common.cuh"
 
 namespace deoct {
@@ -94,7 +96,9 @@ int slice_bits(int W, uint32_t max_nu);            // planes that hold every the
 bool slice_choose(const deoct_ctx* ctx, int D, int F, int K, int P, int nb, int64_t tiles, SliceShape* out);
 int slice_planes(deoct_ctx* ctx, int W, const EvalPlan& plan, const EvalProb* d_probs, int nprob, int64_t tiles,
                  cudaStream_t s);
-int slice_launch(deoct_ctx* ctx, int D, const EvalPlan& plan, const SliceShape& shape, cudaStream_t s);
+// chained: the kernel before it in the stream is the DE step whose trees it evaluates
+int slice_launch(deoct_ctx* ctx, int D, const EvalPlan& plan, const SliceShape& shape, cudaStream_t s,
+                 bool chained = false);
 }  // namespace slc
 
 // CTAs of a re-laid-kernel shape resident on one SM (shared memory and registers;
@@ -158,7 +162,7 @@ struct DEArgs {
   int* part_i = nullptr;
   int* part_g = nullptr;
 };
-enum : int { DE_FIRST = 1, DE_SELECT = 2, DE_TRIAL = 4, DE_GEN_DEVICE = 8 };
+enum : int { DE_FIRST = 1, DE_SELECT = 2, DE_TRIAL = 4, DE_GEN_DEVICE = 8, DE_CHAINED = 16 };
 // The split step: individuals per CTA and lanes per individual, and its scratch
 // (kMaxPop / kDeWideR candidates of 8 + 4 bytes, then the generation number).
 constexpr int kDeWideR = 32, kDeWideG = 8;
@@ -168,7 +172,8 @@ static_assert(kMaxPop / kDeWideR * 12 + 4 <= (int)kDePartBytes, "split-step scra
 int de_launch_init(deoct_ctx* ctx, const DEArgs& a, cudaStream_t s);
 // flags: DE_FIRST (fitness of the evaluated initial population), DE_SELECT
 // (fitness of the evaluated trials + Eq. selection), DE_TRIAL (trial vectors of
-// generation g), DE_GEN_DEVICE (g read from / advanced in prob.gen).
+// generation g), DE_GEN_DEVICE (g read from / advanced in prob.gen), DE_CHAINED (may
+// start before the kernel ahead of it, the evaluation, has ended).
 int de_launch_step(deoct_ctx* ctx, const DEArgs& a, int g, int flags, cudaStream_t s);
 // decode the best individual: a_out [B], theta_out [B], *fit_out (device)
 int launch_best_extract(deoct_ctx* ctx, const float* pop, const double* fit, const int32_t* best,
@@ -213,6 +218,10 @@ int radix_sort_segments(deoct_ctx* ctx, uint32_t* k0, uint32_t* v0, uint32_t* k1
 int engine_generations(deoct_engine* e, const void* owner, int W, int Dt, const DEArgs& a, int G,
                        const std::vector<DEProb>& dp, const std::vector<EvalProb>& ep);
 
+// G generations, each the launches `record` issues on the stream it is given, on
+// stream s: kGensPerGraph of them captured as one graph and replayed, the remainder
+// as another (api.cu).  The graphs may be destroyed once this returns.
+int replay_generations(deoct_ctx* ctx, int G, const std::function<int(cudaStream_t)>& record, cudaStream_t s);
 // the columns of a (sub)set ordered by class (mh.cu); tmp: 3072 bytes of device memory
 int class_order(deoct_ctx* ctx, const deoct_dataset* ds, const int32_t* idx, int64_t n, int32_t* order, void* tmp,
                 cudaStream_t s);

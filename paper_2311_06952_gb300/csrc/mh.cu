@@ -724,8 +724,8 @@ int de_batched(deoct_ctx* ctx, const deoct_dataset* ds, const Compacted& c, uint
     for (const EvalProb& e : be.probs) tiles += slc::slice_tiles(e.count);
     DEOCT_TRY(slc::slice_planes(ctx, W, be.plan, dep, M, tiles, s));
   }
-  auto evaluate = [&](const EvalConfig& cfg, cudaStream_t st) {
-    return sliced ? slc::slice_launch(ctx, Dt, be.plan, sh, st) : eval_launch(ctx, W, Dt, be.plan, cfg, st);
+  auto evaluate = [&](const EvalConfig& cfg, cudaStream_t st, bool chained = false) {
+    return sliced ? slc::slice_launch(ctx, Dt, be.plan, sh, st, chained) : eval_launch(ctx, W, Dt, be.plan, cfg, st);
   };
 
   if (ctx->engine) {
@@ -856,45 +856,19 @@ int de_batched(deoct_ctx* ctx, const deoct_dataset* ds, const Compacted& c, uint
   if (sliced) cfg = scfg;
   DEOCT_TRY(build_plan(ctx, &be, cfg, F, K, P, s));
 
-  // ---- S^1, then G generations from one captured graph ---------------------
+  // ---- S^1, then G generations from captured graphs --------------------------
   DEOCT_TRY(evaluate(cfg, s));
   DEOCT_TRY(de_launch_step(ctx, a, 0, DE_FIRST | DE_GEN_DEVICE | (prm->gens >= 1 ? DE_TRIAL : 0), s));
   if (prm->gens >= 1) {
-    if (!ctx->cap_stream)
-      DEOCT_CUDA_TRY(cudaStreamCreateWithFlags(&ctx->cap_stream, cudaStreamNonBlocking));
-    cudaGraph_t graph = nullptr;
-    cudaGraphExec_t exec = nullptr;
-    const uint64_t l0 = ctx->launches, e0n = ctx->eval_launches;
-    DEOCT_CUDA_TRY(cudaStreamBeginCapture(ctx->cap_stream, cudaStreamCaptureModeThreadLocal));
-    int rc = evaluate(cfg, ctx->cap_stream);
-    if (rc == DEOCT_OK)
-      rc = de_launch_step(ctx, a, 0, DE_SELECT | DE_TRIAL | DE_GEN_DEVICE, ctx->cap_stream);
-    cudaError_t ce = cudaStreamEndCapture(ctx->cap_stream, &graph);
-    if (rc != DEOCT_OK) {
-      if (graph) cudaGraphDestroy(graph);
-      return rc;
-    }
-    if (ce != cudaSuccess)
-      return set_error(DEOCT_ERR_CUDA, "graph capture failed: %s", cudaGetErrorString(ce));
-    const uint64_t per_launch = ctx->launches - l0, per_eval = ctx->eval_launches - e0n;
-    ctx->launches = l0;
-    ctx->eval_launches = e0n;
-    ce = cudaGraphInstantiate(&exec, graph, 0);
-    if (ce != cudaSuccess) {
-      cudaGraphDestroy(graph);
-      return set_error(DEOCT_ERR_CUDA, "graph instantiate failed: %s", cudaGetErrorString(ce));
-    }
-    for (int g = 1; g <= prm->gens; ++g) {
-      ce = cudaGraphLaunch(exec, s);
-      if (ce != cudaSuccess) break;
-      ctx->launches += per_launch;
-      ctx->eval_launches += per_eval;
-    }
-    cudaError_t ce2 = cudaStreamSynchronize(s);
-    cudaGraphExecDestroy(exec);
-    cudaGraphDestroy(graph);
-    if (ce != cudaSuccess) return set_error(DEOCT_ERR_CUDA, "graph launch failed: %s", cudaGetErrorString(ce));
-    if (ce2 != cudaSuccess) return set_error(DEOCT_ERR_CUDA, "generation loop failed: %s", cudaGetErrorString(ce2));
+    DEOCT_TRY(replay_generations(
+        ctx, prm->gens,
+        [&](cudaStream_t st) {
+          DEOCT_TRY(evaluate(cfg, st, true));
+          return de_launch_step(ctx, a, 0, DE_SELECT | DE_TRIAL | DE_GEN_DEVICE | DE_CHAINED, st);
+        },
+        s));
+    const cudaError_t ce = cudaStreamSynchronize(s);
+    if (ce != cudaSuccess) return set_error(DEOCT_ERR_CUDA, "generation loop failed: %s", cudaGetErrorString(ce));
   }
   return extract_roots(ctx, ddp, M, B, ra, rth, rf, s);
 }

@@ -55,3 +55,23 @@ def test_odd_population_in_level_solves(P, K):
     np.testing.assert_array_equal(out["theta"], ref["theta"])
     np.testing.assert_array_equal(out["leaf_class"], ref["leaf_class"])
     ctx.close()
+
+
+@pytest.mark.parametrize("G", [1, 2, 3, 7, 8, 9, 16, 19])
+@pytest.mark.parametrize("P,depth", [(64, 2), (300, 4), (12, 3)])
+def test_generation_graphs(G, P, depth):
+    """Generation counts around the captured graphs' eight, on every step and evaluator kernel."""
+    import torch
+    from paper_2311_06952_gb300 import deoct
+    n, F, K = 1500, 6, 3
+    X, y = _data(G + P, n, F, K)
+    ranks, nu = oracle.encode(X)
+    ref = oracle.de_run(ranks, nu, y, K, depth=depth, P=P, G=G, seed=4)
+    ctx = deoct.Context(0)
+    ds = gpu_dataset(ctx, X, y, K, 2)
+    pop = torch.empty((P, 2 * ((1 << depth) - 1)), dtype=torch.float32, device="cuda")
+    for _ in range(2):
+        _, _, f = deoct.deoct_fit_subtree(ctx, ds, deoct.make_params(depth, P, G, seed=4), pop_out=pop)
+        np.testing.assert_array_equal(pop.cpu().numpy().view(np.uint32), ref["pop"].view(np.uint32))
+        assert f == ref["fit"][ref["best"]]
+    ctx.close()
