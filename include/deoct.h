@@ -126,7 +126,8 @@ DEOCT_API int deoct_reset_stats(deoct_ctx* ctx);
  *  warps  warps per CTA, 1..32 (the streaming kernel, which evaluates groups of
  *         fewer than 16 trees, takes at most 16)
  *  grid   persistent CTAs (each walks an equal contiguous range of tiles)
- * Results do not depend on the shape; only speed does.  Invalid values are
+ * A non-zero value also keeps `ctx` off the bit-sliced evaluator, which has its
+ * own shape.  Results do not depend on the shape; only speed does.  Invalid values are
  * DEOCT_ERR_INVALID; a shape whose tile does not fit in shared memory fails at
  * the next evaluation. */
 DEOCT_API int deoct_set_eval_config(deoct_ctx* ctx, int32_t S, int32_t TG, int32_t warps, int32_t grid);

@@ -1,13 +1,13 @@
-// eval.cu -- population fitness evaluation (Algorithm 1, Section 3.2): the
-// re-laid kernel, the launch decision between it and the streaming kernel
+// eval.cu -- population fitness evaluation (Algorithm 1, Section 3.2) where the
+// bit-sliced evaluator (eval_slice.cuh) is not taken: the re-laid kernel, the launch decision between it and the streaming kernel
 // (eval_stream.cu), and the evaluator's small host-side helpers.
 //
 // The re-laid kernel stages each tile through one landing zone per CTA and,
 // for uint16 ranks, re-lays the rows into a chunk-pair-interleaved compute
 // tile so that 16 warps routing 16+ trees read shared memory without bank
 // conflicts; the next tile's bulk copies fly while the current one is routed.
-// It also holds the shared-atomic counting mode for 2^D K > 128 bins: all
-// warps split each tree's chunks and add into the job's shared counts.
+// It also holds the shared-atomic counting mode for 2^D K > 128 bins: a warp
+// walks one tree's packed nodes over the tile and adds into the job's shared counts.
 #include <cudaTypedefs.h>
 
 #include "eval_kernel.cuh"

@@ -5,14 +5,15 @@
 // the node they reached (node_of); a histogram of (node, class) decides which
 // nodes are solved (more than n_min samples and at least two classes); the
 // samples of solved nodes are compacted into contiguous, 16-sample-aligned
-// segments (sample index, feature-major ranks, labels), so each node's subset
-// is a TMA-able slice; then every solved node is solved with horizon
+// segments (sample index, feature-major ranks, labels; ordered by class inside a
+// segment), so each node's subset is a TMA-able slice; then every solved node is solved with horizon
 // D_t = min(D_MH, D - d):
 //   D_t >= 2: DEOCT of depth D_t (Philox stream = node id), either
 //     - plain: one DEOCT per node, each with its own launches, or
 //     - batched: one multi-problem evaluator launch and one DE-step launch per
-//       generation for all nodes of the level, replayed from a captured CUDA
-//       graph, with the evaluator tile shape chosen by an autotuner;
+//       generation for all nodes of the level, replayed from captured CUDA graphs
+//       of eight generations: the bit-sliced evaluator over the level's bit planes
+//       (level_planes), or the ballot kernels with a shape an autotuner picks;
 //   D_t = 1: exhaustive depth-1 search: per feature, the (node, rank) keys of
 //     the level are radix-sorted so each node's samples are in rank order, and
 //     one CTA per (node, feature) sweeps the distinct ranks with running class

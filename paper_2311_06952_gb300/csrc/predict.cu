@@ -5,7 +5,8 @@
 // (theta+1)-th smallest distinct training values (1-based), computed in double
 // (exact for float32 inputs); theta = 0 is beta_{p,1} = 0 after min-max
 // scaling, i.e. the smallest training value.  On training samples "x < b"
-// then routes exactly like "rank < theta".
+// then routes exactly like "rank < theta".  Many rows of deep trees go through
+// shared-memory tiles (predict_tile_kernel), others are walked a thread a row.
 #include <algorithm>
 
 #include "internal.cuh"
