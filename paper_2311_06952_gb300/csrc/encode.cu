@@ -336,7 +336,7 @@ __global__ void __launch_bounds__(kThreads) rank_scatter_kernel(
   for (int it = 0; it < kItems; ++it) {
     const uint32_t mine = r + __popc(flags[it] & le) - 1u;
     if (j0 + it * 32 + lane < n) {
-      out[val[it]] = (RT)mine;
+      if (val[it] < n) out[val[it]] = (RT)mine;  // (a place below n unless a wait of the sort ran out)
       if (uniq && ((flags[it] >> lane) & 1u)) uniq[(int64_t)f * ld + mine] = from_orderable(key[it]);
     }
     r += __popc(flags[it]);
