@@ -114,7 +114,9 @@ __global__ void __launch_bounds__(kTileThreads) predict_tile_kernel(
   int z = 0;
   uint32_t ph = 0;
   for (int64_t t = blockIdx.x; t < tiles; t += gridDim.x) {
-    if (!mbar_wait_bounded(&full[z], ph, status)) {  // recorded; one more bounded wait for copies in flight
+    // Ran out for a lane: recorded, one more bounded wait for copies in flight.  A warp
+    // leaves as a whole: its lanes meet again in the sum below.
+    if (__any_sync(0xFFFFFFFFu, !mbar_wait_bounded(&full[z], ph, status))) {
       mbar_wait_bounded(&full[z], ph, status);
       break;
     }
