@@ -42,9 +42,9 @@ WORKLOAD = dict(workload="large-deoct: n=1e7, F=10 U(0,1) quantised to 60000 lev
 INT32_LANES_PER_SM = 128  # Blackwell SM: 4 partitions x 32 lanes issue INT32
 # DRAM bytes (read + write) of one evaluator launch on this workload, from an ncu
 # capture of the evaluator on this workload; valid only for the kernel code it was
-# taken on: a hash of the re-laid evaluator kernel's code in csrc/eval.cu and of the
-# headers it is built from (eval_kernel.cuh, common.cuh), comments and whitespace
-# left out.
+# taken on: a hash of the bit-sliced evaluator's code (eval_slice.cu, eval_slice.cuh), of
+# the re-laid kernel's and its shape chooser in csrc/eval.cu and of the headers both are
+# built from (eval_kernel.cuh, common.cuh), comments and whitespace left out.
 EVAL_TRAFFIC = {"source_sha256_16": "4c2a85aa0dc07e19", "bytes": 212_132_864 + 3_597_568,
                 # the same capture: issue rate (of 4 per SM per cycle), pipe and DRAM figures
                 "ncu": {"inst_per_cycle": 3.4608, "issue_frac": 0.8652, "alu_pipe_frac": 0.8130,
@@ -78,8 +78,9 @@ def _strip_comments(src):
 
 
 def _eval_source_hash():
-    """Key of the evaluator kernel's code and launch shape: the `eval_kernel` template and the
-    shape chooser `eval_choose_config` of csrc/eval.cu, the kernel header csrc/eval_kernel.cuh
+    """Key of the evaluators' code and launch shape: the bit-sliced kernel and its chooser
+    (csrc/eval_slice.cu, csrc/eval_slice.cuh), the `eval_kernel` template and the shape
+    chooser `eval_choose_config` of csrc/eval.cu, the kernel header csrc/eval_kernel.cuh
     and the device helpers of csrc/common.cuh (from its "device helpers" section on: the
     host-side context and error code above it are not the kernel's), comments and whitespace
     left out."""
@@ -94,8 +95,9 @@ def _eval_source_hash():
     a = ev.index("EvalConfig eval_choose_config(")
     b = ev.index("\n}\n", a)
     h.update(_strip_comments(ev[a:b]).encode())
-    with open(os.path.join(csrc, "eval_kernel.cuh")) as fh:
-        h.update(_strip_comments(fh.read()).encode())
+    for name in ("eval_slice.cu", "eval_slice.cuh", "eval_kernel.cuh"):
+        with open(os.path.join(csrc, name)) as fh:
+            h.update(_strip_comments(fh.read()).encode())
     with open(os.path.join(csrc, "common.cuh")) as fh:
         common = fh.read()
     h.update(_strip_comments(common[common.index("// device helpers"):]).encode())
@@ -778,7 +780,7 @@ def run_ours(args):
                      "frac": achieved / peak,
                      "traffic": args.traffic if args.traffic is not None else (
                          _traffic_default() if args.n == WORKLOAD["n"] else None),
-                     "kernel": "eval_kernel<2,4,0> (population evaluator)",
+                     "kernel": "eval_slice_kernel<4,ND,false> (bit-sliced population evaluator)",
                      "ops_per_launch": ops_per_launch, "ops_per_eval": ops_per_eval,
                      "launch_ms": eval_ms, "launches_timed": int(st_roof["eval_timed"]),
                      "timing_pass": "one extra step after the timed loop, launches issued directly "
