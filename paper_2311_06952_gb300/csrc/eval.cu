@@ -1,6 +1,7 @@
 // eval.cu -- population fitness evaluation (Algorithm 1, Section 3.2) where the
-// bit-sliced evaluator (eval_slice.cuh) is not taken: the re-laid kernel, the launch decision between it and the streaming kernel
-// (eval_stream.cu), and the evaluator's small host-side helpers.
+// bit-sliced evaluator (eval_slice.cuh) is not taken: the re-laid kernel, the
+// launch decision between it and the streaming kernel (eval_stream.cu), and the
+// evaluator's small host-side helpers.
 //
 // The re-laid kernel stages each tile through one landing zone per CTA and,
 // for uint16 ranks, re-lays the rows into a chunk-pair-interleaved compute
