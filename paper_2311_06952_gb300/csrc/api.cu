@@ -377,8 +377,8 @@ int run_deoct(deoct_ctx* ctx, const deoct_dataset* ds, const int32_t* idx, int64
   return replay_generations(
       ctx, p->gens,
       [&](cudaStream_t st) {
-        DEOCT_TRY(evaluate(st, true));
-        return de_launch_step(ctx, a, 0, DE_SELECT | DE_TRIAL | DE_GEN_DEVICE | DE_CHAINED, st);
+        DEOCT_TRY(evaluate(st, false));
+        return de_launch_step(ctx, a, 0, DE_SELECT | DE_TRIAL | DE_GEN_DEVICE, st);
       },
       s);
 }

@@ -200,25 +200,7 @@ int rebuild(deoct_engine* e, const EngineGroupKey& k, Group& g) {
     mx = std::max(mx, counts[m]);
   }
   deoct_ctx* c = e->ctx;
-  // the bit-sliced evaluator when every problem is set up for it and the mix suits it
-  int nb = 1;
-  int64_t tiles = 0;
-  bool sliced = true;
-  for (int m = 0; m < M; ++m) {
-    sliced = sliced && ep[m].nb > 0 && (ep[m].planes != nullptr) == (ep[0].planes != nullptr);
-    nb = std::max(nb, ep[m].nb);
-    tiles += slc::slice_tiles(counts[m]);
-  }
-  slc::SliceShape sh;
-  sliced = sliced && slc::slice_choose(c, k.Dt, Fmax, Kmax, k.P, nb, tiles, &sh);
-  sh.raw = M > 0 && ep[0].planes == nullptr;
-  EvalConfig cfg;
-  if (sliced) {
-    cfg.S = 1024;
-    cfg.TG = sh.TG;
-  } else {
-    cfg = eval_choose_config(c, k.W, k.Dt, Fmax, Kmax, k.P, std::max<int64_t>(1, nsum), M);
-  }
+  const EvalConfig cfg = eval_choose_config(c, k.W, k.Dt, Fmax, Kmax, k.P, std::max<int64_t>(1, nsum), M);
   std::vector<EvalJob> jobs;
   int64_t total = 0;
   eval_build_jobs(counts, std::vector<int>(M, k.P), cfg.S, cfg.TG, &jobs, &total);
@@ -259,10 +241,8 @@ int rebuild(deoct_engine* e, const EngineGroupKey& k, Group& g) {
   const uint64_t l0 = c->launches, v0 = c->eval_launches;
   cudaGraph_t graph = nullptr;
   DEOCT_CUDA_TRY(cudaStreamBeginCapture(c->cap_stream, cudaStreamCaptureModeThreadLocal));
-  int rc = sliced ? slc::slice_launch(c, k.Dt, plan, sh, c->cap_stream)
-                  : eval_launch(c, k.W, k.Dt, plan, cfg, c->cap_stream);
-  if (rc == DEOCT_OK)
-    rc = de_launch_step(c, a, 0, DE_SELECT | DE_TRIAL | DE_GEN_DEVICE | DE_CHAINED, c->cap_stream);
+  int rc = eval_launch(c, k.W, k.Dt, plan, cfg, c->cap_stream);
+  if (rc == DEOCT_OK) rc = de_launch_step(c, a, 0, DE_SELECT | DE_TRIAL | DE_GEN_DEVICE, c->cap_stream);
   cudaError_t ce = cudaStreamEndCapture(c->cap_stream, &graph);
   g.per_replay_launches = c->launches - l0;
   g.per_replay_evals = c->eval_launches - v0;

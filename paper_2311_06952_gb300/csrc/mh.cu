@@ -889,8 +889,8 @@ int de_batched(deoct_ctx* ctx, const deoct_dataset* ds, const Compacted& c, uint
     DEOCT_TRY(replay_generations(
         ctx, prm->gens,
         [&](cudaStream_t st) {
-          DEOCT_TRY(evaluate(cfg, st, true));
-          return de_launch_step(ctx, a, 0, DE_SELECT | DE_TRIAL | DE_GEN_DEVICE | DE_CHAINED, st);
+          DEOCT_TRY(evaluate(cfg, st, false));
+          return de_launch_step(ctx, a, 0, DE_SELECT | DE_TRIAL | DE_GEN_DEVICE, st);
         },
         s));
     const cudaError_t ce = cudaStreamSynchronize(s);
