@@ -354,7 +354,9 @@ DEOCT_API int deoct_release_scratch(deoct_ctx* ctx);
  * whose scratch would grow past the cap fails with DEOCT_ERR_OOM before it
  * allocates or launches anything for that buffer; the context stays usable (raise
  * the cap, or release scratch, and call again).  Buffers already held above a
- * lowered cap are kept.  sync. */
+ * lowered cap are kept.  Memory that only makes a fit faster (its bit planes) is
+ * left out where the cap leaves no room for it, and given up when a later
+ * request needs the room.  sync. */
 DEOCT_API int deoct_set_scratch_limit(deoct_ctx* ctx, uint64_t bytes);
 DEOCT_API int deoct_fit_scratch_bound(const deoct_ctx* ctx, int64_t n, int32_t F, int32_t K,
                                       int32_t rank_bytes, const deoct_params* params,

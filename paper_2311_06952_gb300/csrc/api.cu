@@ -28,38 +28,79 @@ int check_launch(const char* what) {
   return DEOCT_OK;
 }
 
-int scratch_get(deoct_ctx* ctx, int slot, size_t bytes, void** out) {
+// Grow a slot to `bytes` and up to `head` more: of what the limit leaves at most half,
+// so that one buffer's headroom does not take the room the next buffers need.
+static int scratch_grow(deoct_ctx* ctx, int slot, size_t bytes, size_t head) {
   Scratch& s = ctx->scratch[slot];
-  if (bytes == 0) bytes = 16;
-  if (s.bytes < bytes) {
-    size_t want = bytes + bytes / 8;  // headroom against repeated growth
-    if (ctx->scratch_limit) {  // the buffer's growth must keep the total within the limit
-      size_t others = 0;
-      for (int i = 0; i < SL_COUNT; ++i)
-        if (i != slot) others += ctx->scratch[i].bytes;
-      if (others + bytes > ctx->scratch_limit)
-        return set_error(DEOCT_ERR_OOM,
-                         "scratch of %zu bytes would pass the context's limit of %zu bytes (%zu held "
-                         "in other buffers)", bytes, (size_t)ctx->scratch_limit, others);
-      want = std::min(want, (size_t)ctx->scratch_limit - others);
-    }
-    if (s.ptr) {
-      DEOCT_CUDA_TRY(cudaFree(s.ptr));  // synchronises the device: no pending use
-      s.ptr = nullptr;
-      s.bytes = 0;
-    }
-    cudaError_t e = cudaMalloc(&s.ptr, want);
-    if (e != cudaSuccess) {
-      cudaGetLastError();
-      s.ptr = nullptr;
-      return set_error(DEOCT_ERR_OOM, "scratch allocation of %zu bytes failed: %s", want,
-                       cudaGetErrorString(e));
-    }
-    s.bytes = want;
+  size_t want = bytes + head;
+  if (ctx->scratch_limit) {  // the buffer's growth must keep the total within the limit
+    size_t others = 0;
+    for (int i = 0; i < SL_COUNT; ++i)
+      if (i != slot) others += ctx->scratch[i].bytes;
+    if (others + bytes > ctx->scratch_limit)
+      return set_error(DEOCT_ERR_OOM,
+                       "scratch of %zu bytes would pass the context's limit of %zu bytes (%zu held "
+                       "in other buffers)", bytes, (size_t)ctx->scratch_limit, others);
+    want = bytes + std::min(head, ((size_t)ctx->scratch_limit - others - bytes) / 2);
   }
-  *out = s.ptr;
+  if (s.ptr) {
+    DEOCT_CUDA_TRY(cudaFree(s.ptr));  // synchronises the device: no pending use
+    s.ptr = nullptr;
+    s.bytes = 0;
+  }
+  cudaError_t e = cudaMalloc(&s.ptr, want);
+  if (e != cudaSuccess) {
+    cudaGetLastError();
+    s.ptr = nullptr;
+    return set_error(DEOCT_ERR_OOM, "scratch allocation of %zu bytes failed: %s", want,
+                     cudaGetErrorString(e));
+  }
+  s.bytes = want;
   return DEOCT_OK;
 }
+
+int scratch_get(deoct_ctx* ctx, int slot, size_t bytes, void** out) {
+  const uint64_t bit = uint64_t(1) << slot;
+  if (bytes == 0) bytes = 16;
+  if (ctx->scratch[slot].bytes < bytes) {
+    int rc = scratch_grow(ctx, slot, bytes, bytes / 8);  // headroom against repeated growth
+    const uint64_t idle = ctx->optional & ~ctx->optional_used & ~bit;
+    if (rc == DEOCT_ERR_OOM && idle) {
+      clear_error();
+      for (int i = 0; i < SL_COUNT; ++i)
+        if ((idle >> i) & 1) {
+          DEOCT_CUDA_TRY(cudaFree(ctx->scratch[i].ptr));  // synchronises the device
+          ctx->scratch[i].ptr = nullptr;
+          ctx->scratch[i].bytes = 0;
+        }
+      ctx->optional &= ~idle;
+      rc = scratch_grow(ctx, slot, bytes, bytes / 8);
+    }
+    if (rc != DEOCT_OK) return rc;
+  }
+  ctx->optional &= ~bit;
+  ctx->optional_used &= ~bit;
+  *out = ctx->scratch[slot].ptr;
+  return DEOCT_OK;
+}
+
+bool scratch_try(deoct_ctx* ctx, int slot, size_t bytes, void** out) {
+  const uint64_t bit = uint64_t(1) << slot;
+  if (bytes == 0) bytes = 16;
+  if (ctx->scratch[slot].bytes < bytes) {
+    // under a limit no headroom: what is left is for what calls need
+    if (scratch_grow(ctx, slot, bytes, ctx->scratch_limit ? 0 : bytes / 8) != DEOCT_OK) {
+      clear_error();
+      return false;
+    }
+    ctx->optional |= bit;
+  }
+  ctx->optional_used |= bit;
+  *out = ctx->scratch[slot].ptr;
+  return true;
+}
+
+void scratch_done(deoct_ctx* ctx, int slot) { ctx->optional_used &= ~(uint64_t(1) << slot); }
 
 int pinned_get(deoct_ctx* ctx, size_t bytes, void** out) {
   if (ctx->h_pinned_bytes < bytes) {
@@ -179,21 +220,15 @@ static int slice_planes_of_fit(deoct_ctx* ctx, const deoct_dataset* ds, const in
   const size_t bytes = slc::slice_plane_bytes(slc::slice_tiles(n_sub), ds->F, ds->K, p.nb);
   if (bytes > std::max(ctx->scratch[SL_ENC_K0].bytes, 4 * (size_t)n_sub * ds->F)) return DEOCT_OK;
   uint32_t* buf = nullptr;
-  if (scratch_get(ctx, SL_ENC_K0, bytes, (void**)&buf) != DEOCT_OK) {
-    clear_error();
-    return DEOCT_OK;
-  }
+  if (!scratch_try(ctx, SL_ENC_K0, bytes, (void**)&buf)) return DEOCT_OK;
   const size_t order_bytes = 3072 + sizeof(int32_t) * (size_t)n_sub;
   unsigned char* order = nullptr;
   if (ds->K > 1 && tiles >= 2 * ds->K &&
-      order_bytes <= std::max(ctx->scratch[SL_ENC_K1].bytes, 4 * (size_t)n_sub * ds->F)) {
-    if (scratch_get(ctx, SL_ENC_K1, order_bytes, (void**)&order) == DEOCT_OK) {
-      DEOCT_TRY(class_order(ctx, ds, idx, n_sub, reinterpret_cast<int32_t*>(order + 3072), order, s));
-      p.idx = reinterpret_cast<int32_t*>(order + 3072);
-      p.tma = p.lab_tma = 0;
-    } else {
-      clear_error();
-    }
+      order_bytes <= std::max(ctx->scratch[SL_ENC_K1].bytes, 4 * (size_t)n_sub * ds->F) &&
+      scratch_try(ctx, SL_ENC_K1, order_bytes, (void**)&order)) {
+    DEOCT_TRY(class_order(ctx, ds, idx, n_sub, reinterpret_cast<int32_t*>(order + 3072), order, s));
+    p.idx = reinterpret_cast<int32_t*>(order + 3072);
+    p.tma = p.lab_tma = 0;
   }
   p.planes = buf;
   return slc::slice_planes(ctx, ds->rank_bytes, *plan, nullptr, 1, tiles, s);
@@ -350,6 +385,7 @@ int run_deoct(deoct_ctx* ctx, const deoct_dataset* ds, const int32_t* idx, int64
     max_nu = *std::max_element(h, h + ds->F);
   }
   const bool sliced = slice_plan(ctx, ds, idx, n_sub, p->pop, p->depth, max_nu, &sp, &sh);
+  PlaneMemory planes(ctx);  // until this returns; nothing below needs more scratch
   if (sliced) {
     sp.single.nodes = b.nodes;
     sp.single.counts = b.counts;
@@ -570,6 +606,7 @@ int deoct_release_scratch(deoct_ctx* ctx) {
       ctx->scratch[i].ptr = nullptr;
       ctx->scratch[i].bytes = 0;
     }
+  ctx->optional = ctx->optional_used = 0;
   return DEOCT_OK;
   API_END
 }

@@ -106,6 +106,9 @@ struct deoct_ctx {
   int force_S = 0, force_TG = 0, force_warps = 0, force_grid = 0;
   int force_stream = 0;  // deoct_set_eval_streaming: streaming kernel for every ballot launch
   uint64_t scratch_limit = 0;  // deoct_set_scratch_limit: cap of the scratch held (0: none)
+  // buffers that scratch_try grew (bit per slot), and those of them a call is using:
+  // scratch_get frees the others when it would fail without
+  uint64_t optional = 0, optional_used = 0;
   // shared engine that runs the generations of this context's batched level
   // solves together with other contexts' (deoct_engine_attach; nullable)
   deoct_engine* engine = nullptr;
@@ -115,6 +118,13 @@ namespace deoct {
 
 // grow-only device scratch; contents are not preserved on growth
 int scratch_get(deoct_ctx* ctx, int slot, size_t bytes, void** out);
+// The same for memory a call can do without (one that is only faster with it): false,
+// without an error, where the scratch limit or the device leaves no room.  In use until
+// scratch_done, or until scratch_get takes the slot; after that a scratch_get that
+// finds no room frees it.  What a call needs it takes before what it can do without.
+bool scratch_try(deoct_ctx* ctx, int slot, size_t bytes, void** out);
+void scratch_done(deoct_ctx* ctx, int slot);
+static_assert(SL_COUNT <= 64, "a bit per slot");
 // pinned host buffer for read-backs (grow-only)
 int pinned_get(deoct_ctx* ctx, size_t bytes, void** out);
 // read, clear and translate the device status word (sync on `stream`)

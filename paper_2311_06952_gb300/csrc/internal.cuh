@@ -101,6 +101,19 @@ int slice_launch(deoct_ctx* ctx, int D, const EvalPlan& plan, const SliceShape& 
                  bool chained = false);
 }  // namespace slc
 
+// A fit's hold on the memory of its planes and their order (scratch_try).
+struct PlaneMemory {
+  deoct_ctx* ctx;
+  explicit PlaneMemory(deoct_ctx* c) : ctx(c) {}
+  ~PlaneMemory() { done(); }
+  PlaneMemory(const PlaneMemory&) = delete;
+  PlaneMemory& operator=(const PlaneMemory&) = delete;
+  void done() {
+    scratch_done(ctx, SL_ENC_K0);
+    scratch_done(ctx, SL_ENC_K1);
+  }
+};
+
 // CTAs of a re-laid-kernel shape resident on one SM (shared memory and registers;
 // 0 when the shape does not fit or runs on the streaming kernel).
 int eval_ctas_per_sm(const deoct_ctx* ctx, int W, int D, int F, int K, const EvalConfig& c);

@@ -563,12 +563,10 @@ struct BatchedEval {
   EvalPlan plan;
 };
 
-// The bit-sliced evaluator's shape for a level's problems, with memory for their
-// planes in the encoder's first buffer (4 n F bytes in a context that encoded the
-// set, and no fit reads it; without it the evaluator transposes the ranks in
-// every launch).  False: the other kernels evaluate the level.
-bool level_planes(deoct_ctx* ctx, const deoct_dataset* ds, BatchedEval* be, int P, int Dt, uint32_t max_nu,
-                  slc::SliceShape* sh) {
+// The bit-sliced evaluator's shape for a level's problems; false: the other kernels
+// evaluate the level.
+bool level_slice(deoct_ctx* ctx, const deoct_dataset* ds, BatchedEval* be, int P, int Dt, uint32_t max_nu,
+                 slc::SliceShape* sh) {
   if (P < 16) return false;
   const int nb = slc::slice_bits(ds->rank_bytes, max_nu);
   int64_t tiles = 0;
@@ -586,16 +584,21 @@ bool level_planes(deoct_ctx* ctx, const deoct_dataset* ds, BatchedEval* be, int 
     e.nb = nb;
     e.W = ds->rank_bytes;
   }
-  const size_t bytes = slc::slice_plane_bytes(tiles, ds->F, ds->K, nb);
+  return true;
+}
+
+// Memory for the planes of a level's problems: the encoder's first buffer (4 n F bytes
+// in a context that encoded the set, and no fit reads it).  Without it the evaluator
+// transposes the ranks in every launch.
+void level_planes(deoct_ctx* ctx, const deoct_dataset* ds, BatchedEval* be, slc::SliceShape* sh) {
+  const int nb = be->probs[0].nb;
+  const EvalProb& last = be->probs.back();
+  const size_t bytes = slc::slice_plane_bytes(last.ptile0 + slc::slice_tiles(last.count), ds->F, ds->K, nb);
   uint32_t* planes = nullptr;
-  if (bytes > std::max(ctx->scratch[SL_ENC_K0].bytes, 4 * (size_t)ds->n * ds->F)) return true;
-  if (scratch_get(ctx, SL_ENC_K0, bytes, (void**)&planes) != DEOCT_OK) {  // past the scratch limit
-    clear_error();
-    return true;
-  }
+  if (bytes > std::max(ctx->scratch[SL_ENC_K0].bytes, 4 * (size_t)ds->n * ds->F)) return;
+  if (!scratch_try(ctx, SL_ENC_K0, bytes, (void**)&planes)) return;
   sh->raw = false;
   for (EvalProb& e : be->probs) e.planes = planes + slc::slice_plane_bytes(e.ptile0, ds->F, ds->K, nb) / 4;
-  return true;
 }
 
 int build_plan(deoct_ctx* ctx, BatchedEval* be, const EvalConfig& cfg, int F, int K, int P,
@@ -721,10 +724,19 @@ int de_batched(deoct_ctx* ctx, const deoct_dataset* ds, const Compacted& c, uint
     e.lab_tma = (reinterpret_cast<uintptr_t>(c.clabels + e.start) % 16 == 0) ? 1 : 0;
   }
   slc::SliceShape sh;
-  const bool sliced = level_planes(ctx, ds, &be, P, Dt, max_nu, &sh);
+  const bool sliced = level_slice(ctx, ds, &be, P, Dt, max_nu, &sh);
+  EvalConfig scfg;
+  scfg.S = 1024;
+  scfg.TG = sh.TG;
   DEProb* ddp = nullptr;
   EvalProb* dep = nullptr;
   DEOCT_TRY(upload(ctx, SL_DE_PROBS, dp, &ddp, s));
+  PlaneMemory planes(ctx);
+  if (sliced) {  // the scratch the generations need comes before the planes' memory
+    DEOCT_TRY(scratch_get(ctx, SL_EVAL_PROBS, sizeof(EvalProb) * M, (void**)&dep));
+    DEOCT_TRY(build_plan(ctx, &be, scfg, F, K, P, s));
+    level_planes(ctx, ds, &be, &sh);
+  }
   DEOCT_TRY(upload(ctx, SL_EVAL_PROBS, be.probs, &dep, s));
   be.plan.d_probs = dep;
   DEArgs a;
@@ -741,11 +753,7 @@ int de_batched(deoct_ctx* ctx, const deoct_dataset* ds, const Compacted& c, uint
   a.Kmax = K;
   a.status = ctx->d_status;
   DEOCT_TRY(de_launch_init(ctx, a, s));
-  EvalConfig scfg;
-  scfg.S = 1024;
-  scfg.TG = sh.TG;
-  if (sliced && be.probs[0].planes) {
-    be.plan.Fmax = F;
+  if (sliced && !sh.raw) {
     int64_t tiles = 0;
     for (const EvalProb& e : be.probs) tiles += slc::slice_tiles(e.count);
     DEOCT_TRY(slc::slice_planes(ctx, W, be.plan, dep, M, tiles, s));
@@ -758,7 +766,7 @@ int de_batched(deoct_ctx* ctx, const deoct_dataset* ds, const Compacted& c, uint
     // S^1 and the first trials here, then the G generations in the engine's
     // launches shared with other jobs
     EvalConfig cfg = sliced ? scfg : eval_choose_config(ctx, W, Dt, F, K, P, std::max<int64_t>(1, nsum_of(c, M)), M);
-    DEOCT_TRY(build_plan(ctx, &be, cfg, F, K, P, s));
+    if (!sliced) DEOCT_TRY(build_plan(ctx, &be, cfg, F, K, P, s));
     DEOCT_TRY(evaluate(cfg, s));
     DEOCT_TRY(de_launch_step(ctx, a, 0, DE_FIRST | DE_GEN_DEVICE | (prm->gens >= 1 ? DE_TRIAL : 0), s));
     DEOCT_CUDA_TRY(cudaStreamSynchronize(s));
@@ -880,7 +888,7 @@ int de_batched(deoct_ctx* ctx, const deoct_dataset* ds, const Compacted& c, uint
       DEOCT_CUDA_TRY(cudaMemsetAsync(dp[m].counts, 0, (size_t)P * L * K * 4, s));
   }
   if (sliced) cfg = scfg;
-  DEOCT_TRY(build_plan(ctx, &be, cfg, F, K, P, s));
+  else DEOCT_TRY(build_plan(ctx, &be, cfg, F, K, P, s));
 
   // ---- S^1, then G generations from captured graphs --------------------------
   DEOCT_TRY(evaluate(cfg, s));
@@ -896,6 +904,7 @@ int de_batched(deoct_ctx* ctx, const deoct_dataset* ds, const Compacted& c, uint
     const cudaError_t ce = cudaStreamSynchronize(s);
     if (ce != cudaSuccess) return set_error(DEOCT_ERR_CUDA, "generation loop failed: %s", cudaGetErrorString(ce));
   }
+  planes.done();
   return extract_roots(ctx, ddp, M, B, ra, rth, rf, s);
 }
 

@@ -1,0 +1,74 @@
+"""Memory a fit can do without (the planes of the bit-sliced evaluator) under a context's
+scratch cap: a fit that runs without it runs with it too, again in the same context, with the
+same result and within the cap."""
+import numpy as np
+import pytest
+
+from gpu_helpers import gpu_dataset
+
+pytestmark = pytest.mark.gpu
+
+N, F, K, LEVELS = 40_000, 8, 3, 5000
+PLANES = (N + 1023) // 1024 * (F * 13 + K + 2) * 128  # of the whole set: 13 bits hold LEVELS ranks
+
+
+@pytest.fixture(scope="module")
+def data():
+    from paper_2311_06952_gb300 import deoct
+    rng = np.random.Generator(np.random.PCG64(4711))
+    X = (np.floor(rng.random((N, F)) * LEVELS) / LEVELS).astype(np.float32)
+    y = np.where(X[:, 0] + 0.4 * rng.random(N) < 0.6, 0, rng.integers(1, K, N)).astype(np.uint8)
+    enc = deoct.Context(0)  # the fits' contexts hold nothing of the encoder's
+    ds = gpu_dataset(enc, X, y, K, 2)
+    yield ds
+    enc.close()
+
+
+def _subtree(ctx, ds):
+    from paper_2311_06952_gb300 import deoct
+    return deoct.deoct_fit_subtree(ctx, ds, deoct.make_params(3, 32, 4, seed=2))
+
+
+def _horizon(flags):
+    def fit(ctx, ds):
+        from paper_2311_06952_gb300 import deoct
+        prm = deoct.make_params(4, 32, 4, seed=2, horizon=2, flags=deoct.DEOCT_BATCHED if flags else 0)
+        out = deoct.deoct_fit_moving_horizon(ctx, ds, prm)
+        return out["a"], out["theta"], out["node_fit"]
+    return fit
+
+
+def _with(ds, fit, cap, forced, times=1):
+    from paper_2311_06952_gb300 import deoct
+    ctx = deoct.Context(0)
+    try:
+        if forced:  # a forced launch shape keeps the fit off the bit-sliced evaluator and its planes
+            ctx.set_eval_config(S=512, TG=32)
+        ctx.set_scratch_limit(cap)
+        for _ in range(times):
+            out = fit(ctx, ds)
+            assert cap == 0 or ctx.memory()[0] - 4 <= cap
+        return out, ctx.memory()[0]
+    finally:
+        ctx.close()
+
+
+def _same(got, want):
+    for g, w in zip(got, want):
+        np.testing.assert_array_equal(np.asarray(g), np.asarray(w))
+
+
+@pytest.mark.parametrize("above", [16, 24, 48, 64, 200, 400])
+def test_subtree_fit_with_a_cap_a_little_above_the_planes(data, above):
+    want, held = _with(data, _subtree, 0, True)
+    assert held < 16 * 1024  # what the fit needs without planes
+    got, _ = _with(data, _subtree, PLANES + above * 1024, False, times=2)
+    _same(got, want)
+
+
+@pytest.mark.parametrize("batched", [False, True])
+def test_horizon_fit_with_the_cap_that_suffices_without_planes(data, batched):
+    want, held = _with(data, _horizon(batched), 0, True)
+    _same(_with(data, _horizon(batched), held, True)[0], want)
+    got, _ = _with(data, _horizon(batched), held, False, times=2)
+    _same(got, want)
