@@ -724,7 +724,8 @@ int de_batched(deoct_ctx* ctx, const deoct_dataset* ds, const Compacted& c, uint
     e.lab_tma = (reinterpret_cast<uintptr_t>(c.clabels + e.start) % 16 == 0) ? 1 : 0;
   }
   slc::SliceShape sh;
-  const bool sliced = level_slice(ctx, ds, &be, P, Dt, max_nu, &sh);
+  // (an engine's launches run the ballot kernels, which read no planes)
+  const bool sliced = !ctx->engine && level_slice(ctx, ds, &be, P, Dt, max_nu, &sh);
   EvalConfig scfg;
   scfg.S = 1024;
   scfg.TG = sh.TG;
@@ -765,9 +766,9 @@ int de_batched(deoct_ctx* ctx, const deoct_dataset* ds, const Compacted& c, uint
   if (ctx->engine) {
     // S^1 and the first trials here, then the G generations in the engine's
     // launches shared with other jobs
-    EvalConfig cfg = sliced ? scfg : eval_choose_config(ctx, W, Dt, F, K, P, std::max<int64_t>(1, nsum_of(c, M)), M);
-    if (!sliced) DEOCT_TRY(build_plan(ctx, &be, cfg, F, K, P, s));
-    DEOCT_TRY(evaluate(cfg, s));
+    EvalConfig cfg = eval_choose_config(ctx, W, Dt, F, K, P, std::max<int64_t>(1, nsum_of(c, M)), M);
+    DEOCT_TRY(build_plan(ctx, &be, cfg, F, K, P, s));
+    DEOCT_TRY(eval_launch(ctx, W, Dt, be.plan, cfg, s));
     DEOCT_TRY(de_launch_step(ctx, a, 0, DE_FIRST | DE_GEN_DEVICE | (prm->gens >= 1 ? DE_TRIAL : 0), s));
     DEOCT_CUDA_TRY(cudaStreamSynchronize(s));
     if (prm->gens >= 1) DEOCT_TRY(engine_generations(ctx->engine, ctx, W, Dt, a, prm->gens, dp, be.probs));

@@ -72,3 +72,21 @@ def test_horizon_fit_with_the_cap_that_suffices_without_planes(data, batched):
     _same(_with(data, _horizon(batched), held, True)[0], want)
     got, _ = _with(data, _horizon(batched), held, False, times=2)
     _same(got, want)
+
+
+def test_engine_jobs_take_no_memory_for_planes(data):
+    """A level solve whose generations run in a shared engine's launches, which read no planes,
+    takes no memory for them (and so builds none)."""
+    from paper_2311_06952_gb300 import deoct
+    want, plain = _with(data, _horizon(True), 0, True)
+    eng = deoct.Engine(0)
+    ctx = deoct.Context(0)
+    try:
+        ctx.attach_engine(eng)
+        got = _horizon(True)(ctx, data)
+        held = ctx.memory()[0]
+    finally:
+        ctx.close()
+        eng.close()
+    _same(got, want)
+    assert held < plain + PLANES // 2, (held, plain, PLANES)
