@@ -12,12 +12,7 @@ namespace deoct {
 // ---------------------------------------------------------------------------
 // One subproblem for the evaluator: a sample segment of a rank-encoded set and
 // a population of packed trees whose class counts it accumulates.
-//
-// A multiple of 16 bytes: the evaluators take a problem by value inside their
-// parameters, and with 8 bytes past such a multiple the compiler's code for the
-// ballot kernels was up to 8% slower (n = 1.1e6, F = 10, uint16, 60 trees of depth 4:
-// 93.1 us a launch with 112 or 128 bytes, 100.0 with 136; depth 3, K = 5: 85.9 and 89.4).
-struct alignas(16) EvalProb {
+struct EvalProb {
   const void* ranks;       // [F][ld] uint16 / uint32
   const uint8_t* labels;   // per sample (indexed like rank columns)
   const int32_t* idx;      // nullable: the segment lists column indices idx[start..start+count)
@@ -34,7 +29,7 @@ struct alignas(16) EvalProb {
   // is unused then
   const uint16_t* a16 = nullptr;
   const uint32_t* th32 = nullptr;
-  // bit-sliced evaluator: the problem's planes (tile blocks of F nb + K + 2 rows of 32
+  // bit-sliced evaluator: the problem's planes (tile blocks of F nb + K rows of 32
   // words; nullptr: the evaluator transposes the ranks itself), the planes a feature
   // has (0: not set up for it), the rank width in bytes, and the problem's first tile
   // among those of the launch's problems
@@ -42,7 +37,6 @@ struct alignas(16) EvalProb {
   int64_t ptile0 = 0;
   int32_t nb = 0, W = 0;
 };
-static_assert(sizeof(EvalProb) % 16 == 0, "see above");
 // A job is one tree group of one problem; its tiles are contiguous in the
 // flattened tile order that the persistent CTAs split evenly.
 struct EvalJob {
