@@ -29,7 +29,7 @@ struct EvalProb {
   // is unused then
   const uint16_t* a16 = nullptr;
   const uint32_t* th32 = nullptr;
-  // bit-sliced evaluator: the problem's planes (tile blocks of F nb + K rows of 32
+  // bit-sliced evaluator: the problem's planes (tile blocks of F nb + K + 2 rows of 32
   // words; nullptr: the evaluator transposes the ranks itself), the planes a feature
   // has (0: not set up for it), the rank width in bytes, and the problem's first tile
   // among those of the launch's problems
