@@ -704,26 +704,43 @@ __device__ void finish_single(const EvalArgs& a, uint32_t* sm, size_t sm_bytes) 
     }
     __syncthreads();
     if (a.errors_out) {
-      // a lane per leaf, G lanes per tree: a warp reads consecutive leaves (a thread per
+      // A lane per leaf, G lanes per tree: a warp reads consecutive leaves (a thread per
       // tree read one bank with all its lanes: most of the 210 us of 100 trees of depth 8
-      // on 5000 samples; a warp per tree left 24 lanes of a depth-3 tree idle: 256 trees on
-      // 1e5 samples 37.6 us, now 36.2)
-      constexpr int G = L < 32 ? L : 32, T = 32 / G;  // lanes per tree, trees per warp
-      const int lane = threadIdx.x & 31, nw = blockDim.x >> 5;
-      for (int rw = (threadIdx.x >> 5) * T; rw < nr; rw += nw * T) {
-        const int r = rw + lane / G;
-        uint32_t correct = 0;  // at most n <= 2^24
-        if (r < nr) {
+      // on 5000 samples; a warp per tree left 24 lanes of a depth-3 tree idle).  Two leaves
+      // stay a thread per tree: with lanes the ballot kernel of depth 1 took 53.7 us
+      // against 52.5 (n = 1.1e6, F = 10, uint16, 120 trees).  The loops stay rolled: they
+      // run once.
+      if constexpr (L <= 2) {
+        for (int r = threadIdx.x; r < nr; r += blockDim.x) {
           const uint32_t* c = sm + (int64_t)r * LK;
-          for (int l = lane % G; l < L; l += G) {
+          uint32_t correct = 0;  // at most n <= 2^24
+          for (int l = 0; l < L; ++l) {
             uint32_t mx = 0;
             for (int k = 0; k < K; ++k) mx = max(mx, c[l * K + k]);
             correct += mx;
           }
+          a.errors_out[r0 + r] = (uint32_t)P.count - correct;
         }
+      } else {
+        constexpr int G = L < 32 ? L : 32, T = 32 / G;  // lanes per tree, trees per warp
+        const int lane = threadIdx.x & 31, nw = blockDim.x >> 5;
+        for (int rw = (threadIdx.x >> 5) * T; rw < nr; rw += nw * T) {
+          const int r = rw + lane / G;
+          uint32_t correct = 0;
+          if (r < nr) {
+            const uint32_t* c = sm + (int64_t)r * LK;
+#pragma unroll 1
+            for (int l = lane % G; l < L; l += G) {
+              uint32_t mx = 0;
+#pragma unroll 1
+              for (int k = 0; k < K; ++k) mx = max(mx, c[l * K + k]);
+              correct += mx;
+            }
+          }
 #pragma unroll
-        for (int o = G / 2; o > 0; o >>= 1) correct += __shfl_xor_sync(0xFFFFFFFFu, correct, o);
-        if (r < nr && lane % G == 0) a.errors_out[r0 + r] = (uint32_t)P.count - correct;
+          for (int o = G / 2; o > 0; o >>= 1) correct += __shfl_xor_sync(0xFFFFFFFFu, correct, o);
+          if (r < nr && lane % G == 0) a.errors_out[r0 + r] = (uint32_t)P.count - correct;
+        }
       }
     }
     __syncthreads();
