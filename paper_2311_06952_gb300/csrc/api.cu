@@ -163,6 +163,10 @@ static int validate_params(const deoct_params* p, bool need_pop) {
   return DEOCT_OK;
 }
 
+bool rows_copied(const deoct_dataset* ds, const int32_t* idx) {
+  return idx == nullptr && reinterpret_cast<uintptr_t>(ds->ranks) % 16 == 0 && (ds->ld * ds->rank_bytes) % 16 == 0;
+}
+
 EvalPlan single_eval_plan(const deoct_dataset* ds, const int32_t* idx, int64_t n_sub,
                           const uint32_t* nodes, uint32_t* counts, int P, const EvalConfig& cfg) {
   EvalPlan plan;
@@ -179,9 +183,7 @@ EvalPlan single_eval_plan(const deoct_dataset* ds, const int32_t* idx, int64_t n
   p.F = ds->F;
   p.K = ds->K;
   p.P = P;
-  const bool aligned = (reinterpret_cast<uintptr_t>(ds->ranks) % 16 == 0) &&
-                       ((ds->ld * ds->rank_bytes) % 16 == 0);
-  p.tma = (idx == nullptr && aligned) ? 1 : 0;
+  p.tma = rows_copied(ds, idx) ? 1 : 0;
   p.lab_tma = (p.tma && reinterpret_cast<uintptr_t>(ds->labels) % 16 == 0) ? 1 : 0;
   plan.total_tiles = ((n_sub + cfg.S - 1) / cfg.S) * (int64_t)((P + cfg.TG - 1) / cfg.TG);
   plan.Fmax = ds->F;
@@ -250,7 +252,7 @@ static int64_t width_bound(const deoct_dataset* ds) { return std::min<int64_t>(d
 static int eval_ballot(deoct_ctx* ctx, const deoct_dataset* ds, const int32_t* idx, int64_t n_sub,
                        const uint32_t* nodes, uint32_t* counts, int P, int depth, cudaStream_t s) {
   if (n_sub == 0) return DEOCT_OK;
-  EvalConfig cfg = eval_choose_config(ctx, ds->rank_bytes, depth, ds->F, ds->K, P, n_sub, 1);
+  EvalConfig cfg = eval_choose_config(ctx, ds->rank_bytes, depth, ds->F, ds->K, P, n_sub, 1, rows_copied(ds, idx));
   EvalPlan plan = single_eval_plan(ds, idx, n_sub, nodes, counts, P, cfg);
   return eval_launch(ctx, ds->rank_bytes, depth, plan, cfg, s);
 }
@@ -295,7 +297,7 @@ static int eval_single_fused(deoct_ctx* ctx, const deoct_dataset* ds, const int3
     sp.errors_out = errors_out;
     return slc::slice_launch(ctx, depth, sp, sh, s);
   }
-  EvalConfig cfg = eval_choose_config(ctx, ds->rank_bytes, depth, ds->F, ds->K, P, n_sub, 1);
+  EvalConfig cfg = eval_choose_config(ctx, ds->rank_bytes, depth, ds->F, ds->K, P, n_sub, 1, rows_copied(ds, idx));
   EvalPlan plan = single_eval_plan(ds, idx, n_sub, nullptr, base + 4, P, cfg);
   plan.single.a16 = a;
   plan.single.th32 = theta;

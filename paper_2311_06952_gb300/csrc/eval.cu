@@ -210,8 +210,8 @@ __global__ void __launch_bounds__(1024, 1) eval_kernel(const __grid_constant__ E
       // 100 instructions per 32 samples and tree at depth 8).  GB300, one evaluation
       // (before: all warps on one tree at a time, and the last CTA's errors by one thread
       // a tree): n = 1e6, F = 28, 100 trees of depth 8 580 -> 400 us; n = 3e5, 300 trees of
-      // depth 7 500 -> 286; n = 2e6, K = 29, 32 trees of depth 8 1337 -> 529; n = 5000, 100
-      // trees of depth 8 254 -> 39.
+      // depth 7 453 -> 268; n = 2e6, K = 29, 32 trees of depth 8 1440 -> 405; n = 5000, 100
+      // trees of depth 8 256 -> 34.
       const uint32_t* nodes32 = reinterpret_cast<const uint32_t*>(nodes_s);
       const uint32_t SW = (uint32_t)(S * W);
       const bool own = 2 * jv.ntrees > nw;
@@ -383,7 +383,7 @@ int eval_ctas_per_sm(const deoct_ctx* ctx, int W, int D, int F, int K, const Eva
 }
 
 EvalConfig eval_choose_config(deoct_ctx* ctx, int W, int D, int F, int K, int P, int64_t n,
-                              int nprob) {
+                              int nprob, bool copied) {
   EvalConfig c;
   const int mode = eval_mode(D, K);
   const int limit = std::min(ctx->max_smem_optin, 227 * 1024) - 1024;  // room for static smem
@@ -465,31 +465,46 @@ EvalConfig eval_choose_config(deoct_ctx* ctx, int W, int D, int F, int K, int P,
       }
     }
   } else {
-    // shared-atomic mode: a warp takes a tree, so groups are multiples of the 16
-    // warps where the population and shared memory allow, on the largest tile of
-    // 1024 or 512 samples that leaves room for them beside a second CTA (wide uint32
-    // data would otherwise end at one tree per group and restage each tile once per
-    // tree); fewer trees split a tree's chunks over the warps
-    c.S = 1024;
+    // Shared-atomic mode: a warp takes a tree, so groups are multiples of the 16 warps
+    // where the population and shared memory allow (fewer trees split a tree's chunks
+    // over the warps).  Every group stages each tile again, so take the shape of least
+    // modelled makespan: waves of (tile, group) items over the resident CTAs, an item
+    // costing a unit per sample, tree and level, 10 per sample and feature where rows are
+    // gathered (subsets, unaligned rows; bulk copies hardly count) and 26000 besides; a
+    // CTA alone on its SM is done in 0.75 of the time it takes beside a second.  Fitted
+    // to sweeps of S and TG at sixteen shapes: within 6% of their best.  GB300, us a
+    // launch (before: the larger of two tile sizes that leaves room for 16 trees and a
+    // second CTA, then as many trees as fit beside it):
+    //   F = 22, uint32, 550 trees of depth 6: 3.4e5 rows gathered 1328 -> 560, 6.8e5 copied 911 -> 846;
+    //   F = 28, uint32, 100 trees of depth 8: 5e5 gathered 645 -> 470, 1e6 copied 403 -> 401;
+    //   F = 60, uint32, 1e6 rows, 16 trees of depth 6 486 -> 72; F = 250, 4e5 rows, 64 trees 2982 -> 147;
+    //   F = 12, uint16, 1e5 rows, 40 trees of depth 10, K = 5 135 -> 111.
     c.warps = 16;
-    auto most = [&](int S) {  // trees a group may have
-      int t = std::min(P, 256);
-      while (t > 0 && eval_smem(mode, W, D, S, t, F, K, c.warps) > two_per_sm) --t;
-      return t;
+    double best = -1.0;
+    auto consider = [&](int S, int TG) {
+      const size_t smem = eval_smem(mode, W, D, S, TG, F, K, c.warps);
+      if (smem > (size_t)limit) return;
+      const bool alone = smem > two_per_sm;
+      const int64_t ncta = (int64_t)ctx->num_sms * (alone ? 1 : 2);
+      const double waves = (double)((work(S, TG) + ncta - 1) / ncta) * (alone ? 0.75 : 1.0);
+      const double cost = waves * ((double)S * TG * D + (copied ? 0.0 : 10.0 * S * F) + 26000.0);
+      if (best < 0 || cost < best) {
+        best = cost;
+        c.S = S;
+        c.TG = TG;
+      }
     };
-    int tg = most(1024);
-    if (tg < std::min(P, 16)) {
-      c.S = 512;
-      tg = most(512);
+    for (int S : {2048, 1024, 512, 256, 128})
+      for (int tg = 256; tg >= 16; tg -= 16) {
+        const int groups = (P + tg - 1) / tg;
+        consider(S, std::min(P, ((P + groups - 1) / groups + 15) / 16 * 16));  // groups of one size
+      }
+    if (best < 0) {  // no 16 trees beside any tile
+      c.S = 128;
+      c.TG = 1;
+      for (int S : {2048, 1024, 512, 256, 128})
+        for (int tg : {8, 4, 3, 2, 1}) consider(S, std::min(P, tg));
     }
-    if (tg >= 16) {
-      tg = tg / 16 * 16;
-      const int groups = (P + tg - 1) / tg;
-      tg = std::min(tg, ((P + groups - 1) / groups + 15) / 16 * 16);
-    }
-    c.TG = std::max(1, std::min(tg, P));
-    while (eval_smem(mode, W, D, c.S, c.TG, F, K, c.warps) > (size_t)limit && c.S > 128) c.S /= 2;
-    while (work(c.S, c.TG) < 2 * (int64_t)ctx->num_sms && c.TG > 1) c.TG /= 2;
   }
   if (ctx->force_S) c.S = ctx->force_S;
   if (ctx->force_TG) c.TG = std::min(ctx->force_TG, std::max(1, P));

@@ -117,9 +117,10 @@ struct PlaneMemory {
 // CTAs of a re-laid-kernel shape resident on one SM (shared memory and registers;
 // 0 when the shape does not fit or runs on the streaming kernel).
 int eval_ctas_per_sm(const deoct_ctx* ctx, int W, int D, int F, int K, const EvalConfig& c);
-// Choose S / TG / warps for a workload shape (heuristic, tuned by measurement).
+// Choose S / TG / warps for a workload shape (heuristic, tuned by measurement); copied:
+// the rank rows come by bulk copies (rows_copied), not by a load per rank.
 EvalConfig eval_choose_config(deoct_ctx* ctx, int W, int D, int F, int K, int P, int64_t n,
-                              int nprob);
+                              int nprob, bool copied = true);
 // build the job list for host-side problems (tile counts per problem)
 void eval_build_jobs(const std::vector<int64_t>& counts, const std::vector<int>& pops, int S,
                      int TG, std::vector<EvalJob>* jobs, int64_t* total_tiles);
@@ -128,6 +129,7 @@ void eval_build_jobs(const std::vector<int64_t>& counts, const std::vector<int>&
 // kErrorsInvalid instead
 int launch_errors(deoct_ctx* ctx, const uint32_t* counts, int P, int L, int K, int64_t n_valid,
                   uint32_t* errors, cudaStream_t stream, const int* status = nullptr);
+bool rows_copied(const deoct_dataset* ds, const int32_t* idx);
 // The evaluator plan of one population on one (sub)set of a dataset, for the shape `cfg`:
 // rank rows and labels are staged by bulk copies when the set is the whole dataset and the
 // rows are 16-byte aligned (ranks base and row stride), else gathered with plain loads.

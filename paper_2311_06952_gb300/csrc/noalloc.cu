@@ -97,7 +97,8 @@ extern "C" DEOCT_API int deoct_eval_population_noalloc(const deoct_dataset* ds,
     DEOCT_CUDA_TRY(cudaMemsetAsync(counts, 0, counts_bytes, s));
     DEOCT_TRY(launch_pack_nodes(&ctx, a, theta, (int64_t)P * B, ds->F, nodes, s));
     if (n_sub > 0) {
-      EvalConfig cfg = eval_choose_config(&ctx, ds->rank_bytes, depth, ds->F, ds->K, P, n_sub, 1);
+      EvalConfig cfg = eval_choose_config(&ctx, ds->rank_bytes, depth, ds->F, ds->K, P, n_sub, 1,
+                                          rows_copied(ds, sample_idx));
       EvalPlan plan = single_eval_plan(ds, sample_idx, n_sub, nodes, counts, P, cfg);
       DEOCT_TRY(eval_launch(&ctx, ds->rank_bytes, depth, plan, cfg, s));
     }
