@@ -171,13 +171,15 @@ int launch_predict(deoct_ctx* ctx, const float* X, int64_t m, int F, const uint1
   if (m == 0) return DEOCT_OK;
   const int B = (1 << depth) - 1, L = 1 << depth;
   // The tiles read whole rows, the row walk only the sectors (8 floats) on its path:
-  // tiles where a path touches most of a row.  GB300, us with tiles / with the walk:
-  // 2.75M rows of 28, depth 8: 72 / 107, depth 4: 72 / 80, depth 3: 70 / 74, depth 1:
-  // 70 / 68; 4M rows of 5, depth 6: 64 / 95, depth 2: 56 / 46; 1M rows of 60, depth 8:
-  // 58 / 68, depth 3: 58 / 56; 0.5M rows of 200, depth 5: 88 / 62; 1e5 rows level.
+  // tiles where a path touches most of a row.  GB300, device time in us with the walk /
+  // with tiles, 5.3M rows: F = 16, depth 4 100 / 83; F = 28, depth 4 124 / 101, depth 8
+  // 191 / 114; F = 33, depth 5 149 / 119, depth 6 160 / 123; F = 40, depth 5 165 / 144; F =
+  // 48, depth 3 146 / 160, depth 6 198 / 180; 1.2M rows of 60, depth 8 67 / 59, depth 3 53 /
+  // 53; 7e4 rows level.
   if (m >= 65536 && depth >= 4 && 8 * depth >= F && reinterpret_cast<uintptr_t>(X) % 16 == 0) {
-    int S = 512;
-    while (S > 32 && S * F * 4 > kTileBytes) S /= 2;
+    // a row per thread, or two: with powers of two (128 rows for F = 33 to 64) half the
+    // threads had no row, and F = 33, depth 5 took 159 us against the walk's 149
+    const int S = F <= 16 ? 512 : std::min(256, kTileBytes / (F * 4) / 32 * 32);
     const size_t smem = (size_t)kTileStages * S * F * 4 + (size_t)B * 8 + (size_t)L;
     DEOCT_TRY(set_max_dynamic_smem(ctx, predict_tile_kernel));
     const int grid = (int)std::min<int64_t>((m + S - 1) / S, (int64_t)ctx->num_sms * 2);
