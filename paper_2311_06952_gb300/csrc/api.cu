@@ -394,11 +394,11 @@ int run_deoct(deoct_ctx* ctx, const deoct_dataset* ds, const int32_t* idx, int64
     if (p->gens >= 1) DEOCT_TRY(slice_planes_of_fit(ctx, ds, idx, n_sub, &sp, s));
     sh.raw = sp.single.planes == nullptr;
   }
-  auto evaluate = [&](cudaStream_t st, bool chained) {
-    return sliced ? slc::slice_launch(ctx, p->depth, sp, sh, st, chained)
+  auto evaluate = [&](cudaStream_t st) {
+    return sliced ? slc::slice_launch(ctx, p->depth, sp, sh, st)
                   : eval_ballot(ctx, ds, idx, n_sub, b.nodes, b.counts, p->pop, p->depth, st);
   };
-  DEOCT_TRY(evaluate(s, false));
+  DEOCT_TRY(evaluate(s));
   // The generation number lives on the device (set to 1 by the init kernel and
   // advanced by every trial step), so every generation is the same launches: captured
   // as CUDA graphs and replayed.  With per-launch timing on, the launches are issued
@@ -407,7 +407,7 @@ int run_deoct(deoct_ctx* ctx, const deoct_dataset* ds, const int32_t* idx, int64
   if (p->gens < 1) return DEOCT_OK;
   if (ctx->timing || p->gens < 3) {
     for (int g = 1; g <= p->gens; ++g) {
-      DEOCT_TRY(evaluate(s, false));
+      DEOCT_TRY(evaluate(s));
       DEOCT_TRY(de_launch_step(ctx, a, 0, DE_SELECT | DE_TRIAL | DE_GEN_DEVICE, s));
     }
     return DEOCT_OK;
@@ -415,14 +415,15 @@ int run_deoct(deoct_ctx* ctx, const deoct_dataset* ds, const int32_t* idx, int64
   return replay_generations(
       ctx, p->gens,
       [&](cudaStream_t st) {
-        DEOCT_TRY(evaluate(st, false));
+        DEOCT_TRY(evaluate(st));
         return de_launch_step(ctx, a, 0, DE_SELECT | DE_TRIAL | DE_GEN_DEVICE, st);
       },
       s);
 }
 
-// Generations captured in one graph: a kernel of a graph may start before the one
-// ahead of it has ended (launch_chained), across graph launches it may not.
+// Generations captured in one graph: a generation of a small fit is about 10 us of two
+// kernels, which a graph launch for each does not keep fed (n = 1000, 64 trees of depth
+// 2, G = 100: 1.29 ms with one generation a graph, 1.02 with eight).
 constexpr int kGensPerGraph = 8;
 
 int replay_generations(deoct_ctx* ctx, int G, const std::function<int(cudaStream_t)>& record, cudaStream_t s) {

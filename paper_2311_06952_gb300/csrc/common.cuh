@@ -150,34 +150,9 @@ inline int set_max_dynamic_smem(deoct_ctx* ctx, Kern kern) {
   return DEOCT_OK;
 }
 
-// Launch a kernel; `chained`: it may start before the kernel ahead of it in the
-// stream has ended, and waits for it with chain_wait (programmatic dependent
-// launch: the launch latency and what comes before the wait overlap that kernel's
-// end).
-template <typename... P, typename... A>
-inline cudaError_t launch_chained(bool chained, void (*kern)(P...), int grid, int block, size_t smem, cudaStream_t s,
-                                  A... args) {
-  cudaLaunchAttribute at;
-  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  at.val.programmaticStreamSerializationAllowed = 1;
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)grid);
-  cfg.blockDim = dim3((unsigned)block);
-  cfg.dynamicSmemBytes = smem;
-  cfg.stream = s;
-  cfg.attrs = &at;
-  cfg.numAttrs = chained ? 1 : 0;
-  return cudaLaunchKernelEx(&cfg, kern, static_cast<P>(args)...);
-}
-
 // ---------------------------------------------------------------------------
 // device helpers
 // ---------------------------------------------------------------------------
-// Wait until the kernels this one depends on have ended and their writes are seen
-// (at once in a launch that is not chained); allow the next chained kernel to start.
-__device__ __forceinline__ void chain_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-__device__ __forceinline__ void chain_release() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
-
 __device__ __forceinline__ uint32_t smem_u32(const void* p) {
   return static_cast<uint32_t>(__cvta_generic_to_shared(p));
 }

@@ -358,15 +358,14 @@ constexpr int kStepLanes = 3;          // at most 2^3 lanes an individual
 constexpr int kStepP = 256;            // larger populations are split over CTAs (below)
 
 // nw words of global memory to shared memory (dst 16-byte aligned, src of any
-// alignment), asynchronously as far as src allows, by the whole CTA.  All from L2: a
-// chained launch may start on an SM before the kernels that write src have ended.
+// alignment), asynchronously as far as src allows, by the whole CTA.
 __device__ __forceinline__ void copy_async(uint32_t* dst, const uint32_t* src, int nw) {
   int done = 0;
   if ((reinterpret_cast<uintptr_t>(src) & 15) == 0) {
     done = nw & ~3;
     for (int e = 4 * threadIdx.x; e < done; e += 4 * blockDim.x) cp_async16(dst + e, src + e);
   }
-  for (int e = done + threadIdx.x; e < nw; e += blockDim.x) dst[e] = __ldcg(src + e);
+  for (int e = done + threadIdx.x; e < nw; e += blockDim.x) dst[e] = src[e];
 }
 
 // Index of the least of fit[0..P) (the lowest of equals), by one warp; in the order
@@ -422,13 +421,12 @@ __global__ void __launch_bounds__(1024) de_step_chip_kernel(const DEArgs a, int 
   // ---- loads, then generation g's draws while they are in flight: block q of
   // individual i by thread i nblk + q ----------------------------------------------
   copy_async(nu_s, pb.n_unique, F);
-  chain_wait();  // everything below is the evaluation's or the step's before it
-  const int g = (flags & DE_GEN_DEVICE) ? __ldcg(pb.gen) : g_arg;
+  const int g = (flags & DE_GEN_DEVICE) ? *pb.gen : g_arg;
   copy_async(cnt_s, pb.counts, P * LK);
   copy_async(reinterpret_cast<uint32_t*>(tri_s), reinterpret_cast<const uint32_t*>(pb.trial), P * m);
   copy_async(reinterpret_cast<uint32_t*>(pop_s), reinterpret_cast<const uint32_t*>(pb.pop), P * m);
   asm volatile("cp.async.commit_group;" ::: "memory");
-  const double fr = act ? __ldcg(pb.fit + r) : 0.0;
+  const double fr = act ? pb.fit[r] : 0.0;
   const bool trial = g >= 1 && g <= pb.G;
   if (trial)
     for (int e = tid; e < P * nblk; e += NT) {
@@ -498,9 +496,6 @@ __global__ void __launch_bounds__(1024) de_step_chip_kernel(const DEArgs a, int 
       *pb.best = b;
     }
   }
-  // The next evaluation may start: it sets itself up and builds its first tiles while
-  // the trials are made.  (Not earlier: its CTAs would hold SMs other streams can use.)
-  chain_release();
   if (!trial) return;  // device-driven replay past the last generation (uniform)
   __syncthreads();
 
@@ -666,8 +661,7 @@ int de_launch_step(deoct_ctx* ctx, const DEArgs& a, int g, int flags, cudaStream
     int lg = 0;  // lanes an individual (log2)
     while (lg < kStepLanes && (2 << lg) <= (1 << a.depth) && (a.P << lg) * 2 <= 1024) ++lg;
     DEOCT_TRY(set_max_dynamic_smem(ctx, de_step_chip_kernel));
-    DEOCT_CUDA_TRY(launch_chained((flags & DE_CHAINED) != 0, de_step_chip_kernel, nprob, block_for(a.P << lg), smem, s, a,
-                                  g, flags, lg));
+    de_step_chip_kernel<<<nprob, block_for(a.P << lg), smem, s>>>(a, g, flags, lg);
     count_launch(ctx);
     return check_launch("de_step_chip_kernel");
   }

@@ -139,7 +139,7 @@ int slice_planes(deoct_ctx* ctx, int W, const EvalPlan& plan, const EvalProb* d_
   return check_launch("planes_kernel");
 }
 
-int slice_launch(deoct_ctx* ctx, int D, const EvalPlan& plan, const SliceShape& shape, cudaStream_t s, bool chained) {
+int slice_launch(deoct_ctx* ctx, int D, const EvalPlan& plan, const SliceShape& shape, cudaStream_t s) {
   if (plan.total_tiles <= 0) return DEOCT_OK;
   SliceArgs sa;
   evk::EvalArgs& a = sa.e;
@@ -161,7 +161,6 @@ int slice_launch(deoct_ctx* ctx, int D, const EvalPlan& plan, const SliceShape& 
   a.ticket = plan.d_probs == nullptr ? plan.ticket : nullptr;
   a.counts_out = plan.counts_out;
   a.errors_out = plan.errors_out;
-  sa.chained = chained;
   sa.rows = shape.rows;
   sa.ymask_off = shape.rows * 128;
   sa.rec_off = sa.ymask_off + (plan.Kmax + 1) * 128;

@@ -56,7 +56,6 @@ struct SliceArgs {
   int rows;         // thermometer rows in shared memory
   int ymask_off, rec_off, acc_off, smem_bytes;
   int rec_bytes;    // node records of one warp
-  bool chained;     // launched with programmatic dependence on the kernel before
 };
 
 // Digit counts the kernel is built for, ascending.
@@ -479,7 +478,7 @@ struct Trees {
   __device__ __forceinline__ explicit Trees(const EvalProb& P) : nodes(P.nodes), a16(P.a16), th32(P.th32), F(P.F) {}
 };
 __device__ __forceinline__ uint32_t fetch_node(const Trees& T, int64_t e, int* status) {
-  if (T.a16 == nullptr) return __ldcg(T.nodes + e);  // from L2: a chained launch may share an SM with its writers
+  if (T.a16 == nullptr) return T.nodes[e];
   int av = T.a16[e];
   const uint32_t tv = T.th32[e];
   if (av > T.F || (av > 0 && tv > kThetaMask)) {
@@ -774,11 +773,6 @@ __global__ void __launch_bounds__(kWarps * 32, 1) eval_slice_kernel(const __grid
   const int64_t T = a.total_tiles;
   const int64_t t0 = (int64_t)blockIdx.x * T / gridDim.x;
   const int64_t t1 = (int64_t)(blockIdx.x + 1) * T / gridDim.x;
-  // Chained launches (a fit's generations): the trees and the zeroed counts are the
-  // previous step's; planes, jobs and problems are older, so the first tile is built
-  // before the wait.
-  bool waited = RAW;
-  if (RAW) chain_wait();
   bool fit = true;  // the job's thetas fit the rows (uniform)
   int cur_job = -1, held = 0;  // held: tiles in the 16-bit counts
   evk::JobView jv;
@@ -835,10 +829,6 @@ __global__ void __launch_bounds__(kWarps * 32, 1) eval_slice_kernel(const __grid
       __syncthreads();  // a digit's task reads planes that other warps left
     }
     build_tile<ND, RAW>(&dg, blk, P.F, P.K, P.nb, therm_sa, ymask_sa, &s_classes, lane, warp);
-    if (!waited) {
-      chain_wait();
-      waited = true;
-    }
     // the CTA's next tile on its way to L2 while this one is routed
     if (gt + 1 < t1 && jv.tile + 1 < jv.ntiles) {
       if constexpr (!RAW) {
@@ -858,7 +848,6 @@ __global__ void __launch_bounds__(kWarps * 32, 1) eval_slice_kernel(const __grid
       }
     }
     __syncthreads();
-    if (gt + 1 == t1) chain_release();  // the step that follows may be set up now
     route_tile<D, ND>(&dg, P, jv.tree0, jv.ntrees, accw, therm_sa, ymask_sa, rec, acc, s_classes, a.status,
                       lane, warp);
     ++held;
@@ -874,7 +863,7 @@ template <int D, int ND>
 int launch_slice_t(deoct_ctx* ctx, const SliceArgs& sa, bool raw, int grid, cudaStream_t s) {
   auto* kern = raw ? eval_slice_kernel<D, ND, true> : eval_slice_kernel<D, ND, false>;
   DEOCT_TRY(set_max_dynamic_smem(ctx, kern));
-  DEOCT_CUDA_TRY(launch_chained(sa.chained, kern, grid, kWarps * 32, (size_t)sa.smem_bytes, s, sa));
+  kern<<<grid, kWarps * 32, (size_t)sa.smem_bytes, s>>>(sa);
   count_launch(ctx);
   return check_launch("eval_slice_kernel");
 }

@@ -96,9 +96,7 @@ int slice_bits(int W, uint32_t max_nu);            // planes that hold every the
 bool slice_choose(const deoct_ctx* ctx, int D, int F, int K, int P, int nb, int64_t tiles, SliceShape* out);
 int slice_planes(deoct_ctx* ctx, int W, const EvalPlan& plan, const EvalProb* d_probs, int nprob, int64_t tiles,
                  cudaStream_t s);
-// chained: the kernel before it in the stream is the DE step whose trees it evaluates
-int slice_launch(deoct_ctx* ctx, int D, const EvalPlan& plan, const SliceShape& shape, cudaStream_t s,
-                 bool chained = false);
+int slice_launch(deoct_ctx* ctx, int D, const EvalPlan& plan, const SliceShape& shape, cudaStream_t s);
 }  // namespace slc
 
 // A fit's hold on the memory of its planes and their order (scratch_try).
@@ -177,7 +175,7 @@ struct DEArgs {
   int* part_i = nullptr;
   int* part_g = nullptr;
 };
-enum : int { DE_FIRST = 1, DE_SELECT = 2, DE_TRIAL = 4, DE_GEN_DEVICE = 8, DE_CHAINED = 16 };
+enum : int { DE_FIRST = 1, DE_SELECT = 2, DE_TRIAL = 4, DE_GEN_DEVICE = 8 };
 // The split step: individuals per CTA and lanes per individual, and its scratch
 // (kMaxPop / kDeWideR candidates of 8 + 4 bytes, then the generation number).
 constexpr int kDeWideR = 32, kDeWideG = 8;
@@ -187,8 +185,7 @@ static_assert(kMaxPop / kDeWideR * 12 + 4 <= (int)kDePartBytes, "split-step scra
 int de_launch_init(deoct_ctx* ctx, const DEArgs& a, cudaStream_t s);
 // flags: DE_FIRST (fitness of the evaluated initial population), DE_SELECT
 // (fitness of the evaluated trials + Eq. selection), DE_TRIAL (trial vectors of
-// generation g), DE_GEN_DEVICE (g read from / advanced in prob.gen), DE_CHAINED (may
-// start before the kernel ahead of it, the evaluation, has ended).
+// generation g), DE_GEN_DEVICE (g read from / advanced in prob.gen).
 int de_launch_step(deoct_ctx* ctx, const DEArgs& a, int g, int flags, cudaStream_t s);
 // decode the best individual: a_out [B], theta_out [B], *fit_out (device)
 int launch_best_extract(deoct_ctx* ctx, const float* pop, const double* fit, const int32_t* best,

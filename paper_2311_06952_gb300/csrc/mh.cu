@@ -759,8 +759,8 @@ int de_batched(deoct_ctx* ctx, const deoct_dataset* ds, const Compacted& c, uint
     for (const EvalProb& e : be.probs) tiles += slc::slice_tiles(e.count);
     DEOCT_TRY(slc::slice_planes(ctx, W, be.plan, dep, M, tiles, s));
   }
-  auto evaluate = [&](const EvalConfig& cfg, cudaStream_t st, bool chained = false) {
-    return sliced ? slc::slice_launch(ctx, Dt, be.plan, sh, st, chained) : eval_launch(ctx, W, Dt, be.plan, cfg, st);
+  auto evaluate = [&](const EvalConfig& cfg, cudaStream_t st) {
+    return sliced ? slc::slice_launch(ctx, Dt, be.plan, sh, st) : eval_launch(ctx, W, Dt, be.plan, cfg, st);
   };
 
   if (ctx->engine) {
@@ -898,7 +898,7 @@ int de_batched(deoct_ctx* ctx, const deoct_dataset* ds, const Compacted& c, uint
     DEOCT_TRY(replay_generations(
         ctx, prm->gens,
         [&](cudaStream_t st) {
-          DEOCT_TRY(evaluate(cfg, st, false));
+          DEOCT_TRY(evaluate(cfg, st));
           return de_launch_step(ctx, a, 0, DE_SELECT | DE_TRIAL | DE_GEN_DEVICE, st);
         },
         s));
