@@ -379,14 +379,17 @@ int run_deoct(deoct_ctx* ctx, const deoct_dataset* ds, const int32_t* idx, int64
   DEOCT_TRY(de_launch_init(ctx, a, s));
   EvalPlan sp;
   slc::SliceShape sh;
-  if (max_nu == 0) {
+  // (reading n_p back waits for the stream: not for a fit that the evaluator cannot take
+  // even with one bit a rank)
+  bool sliced = slice_plan(ctx, ds, idx, n_sub, p->pop, p->depth, max_nu ? max_nu : 2, &sp, &sh);
+  if (sliced && max_nu == 0) {
     uint32_t* h = nullptr;
     DEOCT_TRY(pinned_get(ctx, sizeof(uint32_t) * ds->F, (void**)&h));
     DEOCT_CUDA_TRY(cudaMemcpyAsync(h, ds->n_unique, sizeof(uint32_t) * ds->F, cudaMemcpyDeviceToHost, s));
     DEOCT_CUDA_TRY(cudaStreamSynchronize(s));
     max_nu = *std::max_element(h, h + ds->F);
+    sliced = slice_plan(ctx, ds, idx, n_sub, p->pop, p->depth, max_nu, &sp, &sh);
   }
-  const bool sliced = slice_plan(ctx, ds, idx, n_sub, p->pop, p->depth, max_nu, &sp, &sh);
   PlaneMemory planes(ctx);  // until this returns; nothing below needs more scratch
   if (sliced) {
     sp.single.nodes = b.nodes;

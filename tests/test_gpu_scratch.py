@@ -90,3 +90,21 @@ def test_engine_jobs_take_no_memory_for_planes(data):
         eng.close()
     _same(got, want)
     assert held < plain + PLANES // 2, (held, plain, PLANES)
+
+
+@pytest.mark.parametrize("P,depth", [(8, 2), (16, 6)])
+def test_a_fit_on_the_other_kernels_reads_back_only_its_result(P, depth):
+    """Fewer than 16 trees and depth 6 keep a fit off the bit-sliced evaluator: it then has no
+    use for n_p on the host (a wait for the stream), and holds no pinned memory for it."""
+    from paper_2311_06952_gb300 import deoct
+    from gpu_helpers import to_dev
+    n, F = 500, 250
+    rng = np.random.Generator(np.random.PCG64(P + depth))
+    pad = np.zeros((F, deoct.padded_ld(n, 2)), np.uint16)
+    pad[:, :n] = rng.integers(0, 50, (F, n))
+    ds = deoct.DeviceDataset(to_dev(pad), 2, to_dev(np.full(F, 50, np.uint32)), to_dev(rng.integers(0, 2, n).astype(np.uint8)),
+                             n, F, 2)
+    ctx = deoct.Context(0)
+    deoct.deoct_fit_subtree(ctx, ds, deoct.make_params(depth, P, 2, seed=1))
+    assert ctx.memory()[1] < 4 * F
+    ctx.close()
