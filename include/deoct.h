@@ -119,6 +119,9 @@ DEOCT_API int deoct_set_timing(deoct_ctx* ctx, int enable);
 /* Read the counters (sync on pending timing events) / reset them. */
 DEOCT_API int deoct_get_stats(deoct_ctx* ctx, deoct_stats* out);
 DEOCT_API int deoct_reset_stats(deoct_ctx* ctx);
+/* Of the evaluator launches since the last reset, those of the bit-sliced kernel, and
+ * the digits the last of them cut a threshold into (0: none).  Neither synchronises. */
+DEOCT_API int deoct_get_slice_stats(deoct_ctx* ctx, uint64_t* launches, int32_t* digits);
 
 /* Override the evaluator's launch shape (0 keeps the library's choice):
  *  S      samples per shared-memory tile (multiple of 128, 128..8192)

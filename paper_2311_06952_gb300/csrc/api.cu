@@ -435,7 +435,7 @@ int replay_generations(deoct_ctx* ctx, int G, const std::function<int(cudaStream
   for (const int gens : {std::min(G, kGensPerGraph), G % std::min(G, kGensPerGraph)}) {
     if (gens == 0) break;
     const int replays = gens == std::min(G, kGensPerGraph) ? G / gens : 1;
-    const uint64_t l0 = ctx->launches, e0 = ctx->eval_launches;
+    const uint64_t l0 = ctx->launches, e0 = ctx->eval_launches, s0 = ctx->slice_launches;
     cudaGraph_t graph = nullptr;
     cudaGraphExec_t exec = nullptr;
     DEOCT_CUDA_TRY(cudaStreamBeginCapture(ctx->cap_stream, cudaStreamCaptureModeThreadLocal));
@@ -443,8 +443,10 @@ int replay_generations(deoct_ctx* ctx, int G, const std::function<int(cudaStream
     for (int i = 0; i < gens && rc == DEOCT_OK; ++i) rc = record(ctx->cap_stream);
     cudaError_t ce = cudaStreamEndCapture(ctx->cap_stream, &graph);
     const uint64_t per_launch = ctx->launches - l0, per_eval = ctx->eval_launches - e0;
+    const uint64_t per_slice = ctx->slice_launches - s0;
     ctx->launches = l0;
     ctx->eval_launches = e0;
+    ctx->slice_launches = s0;
     if (rc != DEOCT_OK) {
       if (graph) cudaGraphDestroy(graph);
       return rc;
@@ -459,6 +461,7 @@ int replay_generations(deoct_ctx* ctx, int G, const std::function<int(cudaStream
       ce = cudaGraphLaunch(exec, s);
       ctx->launches += per_launch;
       ctx->eval_launches += per_eval;
+      ctx->slice_launches += per_slice;
     }
     // the graph may be destroyed once its launches are queued
     cudaGraphExecDestroy(exec);
@@ -578,8 +581,19 @@ int deoct_reset_stats(deoct_ctx* ctx) {
   ctx->ev_pairs.clear();
   ctx->launches = 0;
   ctx->eval_launches = 0;
+  ctx->slice_launches = 0;
+  ctx->slice_digits = 0;
   ctx->eval_ms = 0.0;
   ctx->eval_timed = 0;
+  return DEOCT_OK;
+  API_END
+}
+
+int deoct_get_slice_stats(deoct_ctx* ctx, uint64_t* launches, int32_t* digits) {
+  API_BEGIN
+  if (!ctx) return set_error(DEOCT_ERR_INVALID, "context is NULL");
+  if (launches) *launches = ctx->slice_launches;
+  if (digits) *digits = ctx->slice_digits;
   return DEOCT_OK;
   API_END
 }

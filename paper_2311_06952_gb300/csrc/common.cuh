@@ -96,6 +96,8 @@ struct deoct_ctx {
   // statistics
   uint64_t launches = 0;
   uint64_t eval_launches = 0;
+  uint64_t slice_launches = 0;  // of which bit-sliced
+  int32_t slice_digits = 0;     // digits of the last of those
   int timing = 0;
   std::vector<cudaEvent_t> ev_pairs;  // start/stop pairs of timed evaluator launches
   double eval_ms = 0.0;

@@ -188,6 +188,8 @@ int slice_launch(deoct_ctx* ctx, int D, const EvalPlan& plan, const SliceShape& 
   }
   DEOCT_TRY(rc);
   ctx->eval_launches += 1;
+  ctx->slice_launches += 1;
+  ctx->slice_digits = shape.nd;
   if (timed) {
     DEOCT_CUDA_TRY(cudaEventRecord(e1, s));
     ctx->ev_pairs.push_back(e0);

@@ -36,7 +36,7 @@ EXPORTED = [
     "deoct_eval_population_noalloc", "deoct_encode_ex", "deoct_split_values", "deoct_predict",
     "deoct_selftest_wait", "deoct_encode_auto", "deoct_engine_create", "deoct_engine_destroy",
     "deoct_engine_attach", "deoct_engine_get_stats", "deoct_get_memory", "deoct_fit_scratch_bound",
-    "deoct_release_scratch", "deoct_set_scratch_limit", "deoct_set_eval_streaming",
+    "deoct_release_scratch", "deoct_set_scratch_limit", "deoct_set_eval_streaming", "deoct_get_slice_stats",
 ]
 NOALLOC_SCRATCH_BYTES = 8 << 20
 
@@ -97,6 +97,7 @@ def load(path: str | None = None):
             "deoct_set_timing": [_vp, ctypes.c_int],
             "deoct_get_stats": [_vp, ctypes.POINTER(Stats)],
             "deoct_reset_stats": [_vp],
+            "deoct_get_slice_stats": [_vp, ctypes.POINTER(_u64), ctypes.POINTER(ctypes.c_int32)],
             "deoct_set_eval_config": [_vp, _i32, _i32, _i32, _i32],
             "deoct_selftest_wait": [_vp, _i32, _vp],
             "deoct_encode": [_vp, _vp, _i64, _i32, _i32, _vp, _i64, _vp, _vp],
@@ -266,6 +267,13 @@ class Context:
         _check(load().deoct_get_stats(self.handle, ctypes.byref(s)))
         return dict(launches=s.launches, eval_launches=s.eval_launches, eval_ms=s.eval_ms,
                     eval_timed=s.eval_timed)
+
+    def slice_stats(self):
+        """(launches of the bit-sliced evaluator since the last reset, digits a threshold had in
+        the last of them; 0: none)."""
+        n, d = _u64(), ctypes.c_int32()
+        _check(load().deoct_get_slice_stats(self.handle, ctypes.byref(n), ctypes.byref(d)))
+        return int(n.value), int(d.value)
 
     def reset_stats(self):
         _check(load().deoct_reset_stats(self.handle))
