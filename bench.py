@@ -112,6 +112,32 @@ def _ncu_default():
     return EVAL_TRAFFIC["ncu"] if _eval_source_hash() == EVAL_TRAFFIC["source_sha256_16"] else None
 
 
+def _eval_roofline(sliced, D, P, n, seconds, nsm, sm_mhz, peak_kind):
+    """The bound of one evaluator launch and the share of it reached.  sliced: (launches of
+    the bit-sliced evaluator, digits a threshold has there).  Its bound is the shared-memory
+    data pipe, one wavefront of 128 bytes a cycle per SM: a node of a tree takes 2 digits - 1
+    rows of 128 bytes for 1024 samples.  Otherwise the ballot kernels' lanes: per tree, sample
+    and level the node's feature and threshold, the sample's rank, the comparison and the step
+    to the child; then the count (2)."""
+    if sliced[0]:
+        rows = 2 * sliced[1] - 1
+        work = -(-n // 1024) * (-(-P // 4) * 4) * ((1 << D) - 1) * rows
+        peak = nsm * sm_mhz * 1e6 / 1e9
+        d = {"bound": "shared", "unit": "Gwavefronts/s", "achieved": work / seconds / 1e9,
+             "kernel": "eval_slice_kernel<%d,%d> (bit-sliced population evaluator)" % (D, sliced[1]),
+             "wavefronts_per_launch": work, "row_loads_per_node": rows,
+             "peak_basis": "%d SMs x 1 wavefront x %.0f MHz (%s max clock)" % (nsm, sm_mhz, peak_kind)}
+    else:
+        ops = 4 * D + 2
+        peak = nsm * INT32_LANES_PER_SM * sm_mhz * 1e6 / 1e12
+        d = {"bound": "alu", "unit": "Tops/s", "achieved": ops * P * n / seconds / 1e12,
+             "kernel": "eval_kernel<2,%d> (ballot population evaluator)" % D,
+             "ops_per_launch": ops * P * n, "ops_per_eval": ops,
+             "peak_basis": "%d SMs x %d INT32 lanes x %.0f MHz (%s max clock)" % (
+                 nsm, INT32_LANES_PER_SM, sm_mhz, peak_kind)}
+    return {**d, "peak": peak, "frac": d["achieved"] / peak, "evals_per_s": P * n / seconds}
+
+
 def _peaks():
     p = os.path.join(ROOT, "MEASURED_PEAKS.json")
     if os.path.exists(p):
@@ -708,7 +734,7 @@ def run_ours(args):
     step(multirank.stream_id(rank))
     f1.record(stream)
     torch.cuda.synchronize()
-    st_roof = ctx.stats()
+    st_roof, slice_roof = ctx.stats(), ctx.slice_stats()
     ctx.set_timing(False)
     ms_step_timed_launches = f0.elapsed_time(f1)
 
@@ -760,15 +786,8 @@ def run_ours(args):
         return 0
     peaks, peak_kind = _peaks()
     eval_ms = st_roof["eval_ms"] / max(1, st_roof["eval_timed"])
-    sm_mhz = float(peaks.get("sm_max_mhz", 2070.0))
-    # per tree-sample evaluation, per level: load the node's feature and threshold, load the
-    # sample's rank, compare, step to the child; then the count increment (2)
-    ops_per_eval = 4 * D + 2
-    ops_per_launch = ops_per_eval * P * n
-    achieved = ops_per_launch / (eval_ms / 1000.0) / 1e12
-    strict_ops = (2 * D + 1) * P * n  # only the comparison and the child step per level, one count
     nsm = torch.cuda.get_device_properties(0).multi_processor_count
-    peak = nsm * INT32_LANES_PER_SM * sm_mhz * 1e6 / 1e12
+    roof = _eval_roofline(slice_roof, D, P, n, eval_ms / 1000.0, nsm, float(peaks.get("sm_max_mhz", 2070.0)), peak_kind)
     bytes_per_launch = n * (F * 2 + 1)
     hbm_achieved = bytes_per_launch / (eval_ms / 1000.0) / 1e9
     line = {
@@ -776,22 +795,14 @@ def run_ours(args):
         "warmup": args.warmup, "ms_per_step": ms_step, "higher_is_better": True, "scaling": "weak",
         "vs_baseline": None, "dtype": "u16", "data": "synthetic",
         "config": w, "gpu_launches": int(st["launches"]),
-        "roofline": {"bound": "alu", "achieved": achieved, "peak": peak, "unit": "Tops/s",
-                     "frac": achieved / peak,
+        "roofline": {**roof,
                      "traffic": args.traffic if args.traffic is not None else (
                          _traffic_default() if args.n == WORKLOAD["n"] else None),
-                     "kernel": "eval_slice_kernel<4,ND,false> (bit-sliced population evaluator)",
-                     "ops_per_launch": ops_per_launch, "ops_per_eval": ops_per_eval,
                      "launch_ms": eval_ms, "launches_timed": int(st_roof["eval_timed"]),
                      "timing_pass": "one extra step after the timed loop, launches issued directly "
                                     "with CUDA events around each evaluator launch (%.1f ms for the "
                                     "step vs %.1f ms per graph-replayed step in the timed loop)"
                                     % (ms_step_timed_launches, ms_step),
-                     "strict_view": {"ops_per_eval": 2 * D + 1, "ops_per_launch": strict_ops,
-                                     "achieved": strict_ops / (eval_ms / 1000.0) / 1e12,
-                                     "frac": strict_ops / (eval_ms / 1000.0) / 1e12 / peak},
-                     "peak_basis": "%d SMs x %d INT32 lanes x %.0f MHz (%s max clock)" % (
-                         nsm, INT32_LANES_PER_SM, sm_mhz, peak_kind),
                      "issue_view": _ncu_default() if args.n == WORKLOAD["n"] else None,
                      "hbm_view": {"achieved_gbs": hbm_achieved, "peak_gbs": peaks["hbm_gbs"],
                                   "frac": hbm_achieved / peaks["hbm_gbs"],
