@@ -141,6 +141,10 @@ DEOCT_API int deoct_set_eval_config(deoct_ctx* ctx, int32_t S, int32_t TG, int32
  * (the batched level solve measures both).  Results are unchanged; 0 restores
  * the automatic choice.  sync. */
 DEOCT_API int deoct_set_eval_streaming(deoct_ctx* ctx, int32_t on);
+/* deoct_set_eval_slicing: where `ctx` evaluates with the bit-sliced kernel (depth <= 5,
+ * 16 trees or more): 0 the library's choice, 1 wherever it can run, -1 nowhere.
+ * Results are the same. */
+DEOCT_API int deoct_set_eval_slicing(deoct_ctx* ctx, int32_t mode);
 
 /* Self-test of the library's failure detection (no counterpart in the paper).
  * Every device-side wait of the library (the evaluator's mbarrier waits) is

@@ -199,7 +199,7 @@ static bool slice_plan(const deoct_ctx* ctx, const deoct_dataset* ds, const int3
                        int depth, int64_t max_nu, EvalPlan* plan, slc::SliceShape* sh) {
   if (n_sub < 1 || P < 16) return false;  // (fewer trees run on the streaming kernel)
   const int W = ds->rank_bytes, nb = slc::slice_bits(W, (uint32_t)max_nu);
-  if (!slc::slice_choose(ctx, depth, ds->F, ds->K, P, nb, slc::slice_tiles(n_sub), sh)) return false;
+  if (!slc::slice_choose(ctx, depth, ds->F, ds->K, P, nb, slc::slice_tiles(n_sub), 0, sh)) return false;
   EvalConfig cfg;
   cfg.S = 1024;
   cfg.TG = sh->TG;
@@ -241,7 +241,9 @@ static int slice_planes_of_fit(deoct_ctx* ctx, const deoct_dataset* ds, const in
 // 145 at n = 1e6, F = 30, depth 3, 49 against 45 at n = 2e5, K = 10; 256 trees 39
 // against 35 us at n = 1e5, F = 20, depth 3, 500 against 790 at n = 2e6, depth 5; 1024
 // trees 4.5 ms against 10.2 at n = 1e7, depth 4).
-static bool slice_once(int64_t n_sub, int P) { return P >= 192 && n_sub * P >= (int64_t(1) << 27); }
+bool slice_once(const deoct_ctx* ctx, int64_t n_sub, int P) {
+  return ctx->force_slice > 0 || (P >= 192 && n_sub * P >= (int64_t(1) << 27));
+}
 
 // Bound of an encoded set's ranks that needs no look at the device: its size, and
 // the rank width.  (Where a set breaks it the evaluator still counts right, slowly.)
@@ -264,7 +266,7 @@ static int eval_single(deoct_ctx* ctx, const deoct_dataset* ds, const int32_t* i
   if (n_sub == 0) return DEOCT_OK;
   EvalPlan sp;
   slc::SliceShape sh;
-  if (slice_once(n_sub, P) && slice_plan(ctx, ds, idx, n_sub, P, depth, width_bound(ds), &sp, &sh)) {
+  if (slice_once(ctx, n_sub, P) && slice_plan(ctx, ds, idx, n_sub, P, depth, width_bound(ds), &sp, &sh)) {
     sp.single.nodes = nodes;
     sp.single.counts = counts;
     return slc::slice_launch(ctx, depth, sp, sh, s);
@@ -288,7 +290,7 @@ static int eval_single_fused(deoct_ctx* ctx, const deoct_dataset* ds, const int3
   if (grows) DEOCT_CUDA_TRY(cudaMemsetAsync(base, 0, ctx->scratch[SL_EVAL_ACC].bytes, s));
   EvalPlan sp;
   slc::SliceShape sh;
-  if (slice_once(n_sub, P) && slice_plan(ctx, ds, idx, n_sub, P, depth, width_bound(ds), &sp, &sh)) {
+  if (slice_once(ctx, n_sub, P) && slice_plan(ctx, ds, idx, n_sub, P, depth, width_bound(ds), &sp, &sh)) {
     sp.single.a16 = a;
     sp.single.th32 = theta;
     sp.single.counts = base + 4;
@@ -379,16 +381,21 @@ int run_deoct(deoct_ctx* ctx, const deoct_dataset* ds, const int32_t* idx, int64
   DEOCT_TRY(de_launch_init(ctx, a, s));
   EvalPlan sp;
   slc::SliceShape sh;
-  // (reading n_p back waits for the stream: not for a fit that the evaluator cannot take
-  // even with one bit a rank)
-  bool sliced = slice_plan(ctx, ds, idx, n_sub, p->pop, p->depth, max_nu ? max_nu : 2, &sp, &sh);
+  // the ballot kernels' modelled time; n_p is read back, which waits for the stream, only
+  // where the bit-sliced evaluator would win with one bit a rank
+  const EvalConfig ballot = eval_choose_config(ctx, ds->rank_bytes, p->depth, ds->F, ds->K, p->pop,
+                                               std::max<int64_t>(1, n_sub), 1, rows_copied(ds, idx));
+  auto wins = [&](int64_t nu) {
+    return slice_plan(ctx, ds, idx, n_sub, p->pop, p->depth, nu, &sp, &sh) && slc::slice_wins(ctx, sh, ballot);
+  };
+  bool sliced = wins(max_nu ? max_nu : 2);
   if (sliced && max_nu == 0) {
     uint32_t* h = nullptr;
     DEOCT_TRY(pinned_get(ctx, sizeof(uint32_t) * ds->F, (void**)&h));
     DEOCT_CUDA_TRY(cudaMemcpyAsync(h, ds->n_unique, sizeof(uint32_t) * ds->F, cudaMemcpyDeviceToHost, s));
     DEOCT_CUDA_TRY(cudaStreamSynchronize(s));
     max_nu = *std::max_element(h, h + ds->F);
-    sliced = slice_plan(ctx, ds, idx, n_sub, p->pop, p->depth, max_nu, &sp, &sh);
+    sliced = wins(max_nu);
   }
   PlaneMemory planes(ctx);  // until this returns; nothing below needs more scratch
   if (sliced) {
@@ -396,6 +403,8 @@ int run_deoct(deoct_ctx* ctx, const deoct_dataset* ds, const int32_t* idx, int64
     sp.single.counts = b.counts;
     if (p->gens >= 1) DEOCT_TRY(slice_planes_of_fit(ctx, ds, idx, n_sub, &sp, s));
     sh.raw = sp.single.planes == nullptr;
+    // without planes every generation transposes the ranks again, as one evaluation does
+    if (sh.raw && !slice_once(ctx, n_sub, p->pop)) sliced = false;
   }
   auto evaluate = [&](cudaStream_t st) {
     return sliced ? slc::slice_launch(ctx, p->depth, sp, sh, st)
@@ -658,6 +667,15 @@ int deoct_set_eval_config(deoct_ctx* ctx, int32_t S, int32_t TG, int32_t warps, 
   ctx->force_TG = TG;
   ctx->force_warps = warps;
   ctx->force_grid = grid;
+  return DEOCT_OK;
+  API_END
+}
+
+int deoct_set_eval_slicing(deoct_ctx* ctx, int32_t mode) {
+  API_BEGIN
+  CTX_CHECK(ctx);
+  if (mode < -1 || mode > 1) return set_error(DEOCT_ERR_INVALID, "mode = %d: want -1, 0 or 1", mode);
+  ctx->force_slice = mode;
   return DEOCT_OK;
   API_END
 }

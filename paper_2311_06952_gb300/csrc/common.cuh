@@ -106,6 +106,7 @@ struct deoct_ctx {
   std::vector<std::pair<uint64_t, std::array<int, 4>>> tuned;  // S, TG, warps, stream
   // evaluator launch shape forced by deoct_set_eval_config (0 = automatic)
   int force_S = 0, force_TG = 0, force_warps = 0, force_grid = 0;
+  int force_slice = 0;   // deoct_set_eval_slicing: 1 wherever it can run, -1 never
   int force_stream = 0;  // deoct_set_eval_streaming: streaming kernel for every ballot launch
   uint64_t scratch_limit = 0;  // deoct_set_scratch_limit: cap of the scratch held (0: none)
   // buffers that scratch_try grew (bit per slot), and those of them a call is using:

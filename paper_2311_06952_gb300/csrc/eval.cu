@@ -456,6 +456,10 @@ EvalConfig eval_choose_config(deoct_ctx* ctx, int W, int D, int F, int K, int P,
             c.warps = 32;
           }
         }
+      // time of a launch in us, fitted to 649 random shapes (see slice_choose; standard
+      // deviation 11%)
+      const int Q = bins_per_lane(D, (1 << D) * K);
+      c.us = best < 0 ? 1e30 : 5.45 + 0.81 * (5 - D) + best * (9.08e-5 * D + 2.43e-5 * (Q - 1));
       if (best < 0) {  // nothing keeps two CTAs per SM: the largest shape that fits
         c.S = 2048;
         c.TG = std::min(P, 256);
@@ -499,6 +503,7 @@ EvalConfig eval_choose_config(deoct_ctx* ctx, int W, int D, int F, int K, int P,
         const int groups = (P + tg - 1) / tg;
         consider(S, std::min(P, ((P + groups - 1) / groups + 15) / 16 * 16));  // groups of one size
       }
+    c.us = best < 0 ? 1e30 : 5.45 + 0.81 * (5 - D) + 1.11e-4 * best;  // (as above, 76 shapes of depth 4 and 5)
     if (best < 0) {  // no 16 trees beside any tile
       c.S = 128;
       c.TG = 1;

@@ -82,9 +82,10 @@ int slice_bits(int W, uint32_t max_nu) {
   return b;
 }
 
-bool slice_choose(const deoct_ctx* ctx, int D, int F, int K, int P, int nb, int64_t tiles, SliceShape* out) {
+bool slice_choose(const deoct_ctx* ctx, int D, int F, int K, int P, int nb, int64_t tiles, int nprob, SliceShape* out) {
   if (D < 1 || D > kMaxDepthSlice || P < 1 || tiles < 1) return false;
-  if (ctx->force_S || ctx->force_TG || ctx->force_warps || ctx->force_grid || ctx->force_stream) return false;
+  if (ctx->force_S || ctx->force_TG || ctx->force_warps || ctx->force_grid || ctx->force_stream || ctx->force_slice < 0)
+    return false;
   const size_t cap = (size_t)std::min(ctx->max_smem_optin, 227 * 1024) - 1024;  // room for static smem
   const int accw = count_words(D, K);
   const size_t ymask = (size_t)(K + 1) * 128;
@@ -101,7 +102,8 @@ bool slice_choose(const deoct_ctx* ctx, int D, int F, int K, int P, int nb, int6
       const int nd = pick_digits(nb, F, rows);
       if (nd == 0 || (nd + 3) / 4 * 16 > rb) continue;
       // Work of one (tile, group): expanding the rows, then the group's trees, in
-      // cycles; waves of them over the SMs (one CTA each).
+      // cycles (weights estimated from phase timings, not fitted: they order the shapes;
+      // the launch's time is modelled below); waves of them over the SMs (one CTA each).
       const double build = 900.0 + 1.3 * F * (digit_rows(nb, nd) + nb);
       const double wf = 4.0 * ((1 << D) - 1) * (2 * nd + 1) + 70.0 * std::max(1, (1 << D) / 8);
       const double quads = tg / 4.0;
@@ -119,7 +121,35 @@ bool slice_choose(const deoct_ctx* ctx, int D, int F, int K, int P, int nb, int6
       break;
     }
   }
-  return best >= 0;
+  if (best < 0) return false;
+  // Time of a launch with planes, us, fitted to 725 random shapes (n = 100 to 1.5e6, F = 4
+  // to 60, 6 to 20 bits, 16 to 1024 trees, depth 1 to 5, K = 2 to 9; standard deviation
+  // 10%): the launch; the constant rows; per wave of items the table from the planes, the
+  // trees' row loads (latency of a warp's quads, then the SM's rate), and the counts of
+  // every class where tiles hold several.
+  const int tg = out->TG, nd = out->nd, ng = (P + tg - 1) / tg, leaves8 = std::max(1, (1 << D) / 8);
+  const double waves = (double)((tiles * ng + ctx->num_sms - 1) / ctx->num_sms);
+  const double quads = tg / 4.0, rounds = std::ceil(quads / kWarps), loads = ((1 << D) - 1) * (2.0 * nd + 1);
+  // classes of a tile: one where the samples are ordered by class, but for the tiles at the
+  // K - 1 borders of a problem; all of them in a set too small to be ordered
+  const int64_t borders = (int64_t)(K - 1) * nprob;
+  const int classes = nprob == 0 ? (tiles >= 2 * K ? 1 : K) : tiles >= 2 * borders ? 1 : (int)std::min<int64_t>(K, 1 + (borders + tiles - 1) / tiles);
+  out->us = 7.28 + 0.0038 * F * nd +
+            waves * (0.595 + 8.2e-4 * F * (digit_rows(nb, nd) + nb) + loads * (0.00996 * rounds + 0.0015 * quads) +
+                     0.2845 * rounds * leaves8 * classes);
+  return true;
+}
+
+// Taken wherever it could run, the bit-sliced evaluator was the slower one at 41% of those
+// 725 shapes, and launches took 13% longer than the better one's on average; by the models
+// 0.8%.  (5% in its favour: the average is the same from 1 to 1.05, and what is lost where
+// the bit-sliced one is the better one falls from 0.5 to 0.2%.)  A generation on the ballot
+// kernels / bit-sliced, us: n = 3e5, F = 38, 20 bits, 128 trees of depth 5 94 / 627 (the rows
+// leave room for four trees a CTA); n = 1000, F = 30, 17 bits, 128 trees of depth 3 10.9 /
+// 14.2; n = 1e5, F = 24, 16 bits, 128 trees of depth 3 25.4 / 18.4; n = 3e5, F = 10, 12 bits,
+// 512 trees of depth 4 181 / 64.
+bool slice_wins(const deoct_ctx* ctx, const SliceShape& s, const EvalConfig& ballot) {
+  return ctx->force_slice > 0 || s.us < 1.05 * ballot.us;
 }
 
 int slice_planes(deoct_ctx* ctx, int W, const EvalPlan& plan, const EvalProb* d_probs, int nprob, int64_t tiles,

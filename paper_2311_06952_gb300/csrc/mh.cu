@@ -563,10 +563,10 @@ struct BatchedEval {
   EvalPlan plan;
 };
 
-// The bit-sliced evaluator's shape for a level's problems; false: the other kernels
-// evaluate the level.
+// The bit-sliced evaluator's shape for a level's problems; false: the other kernels, of
+// modelled time `ballot`, evaluate the level.
 bool level_slice(deoct_ctx* ctx, const deoct_dataset* ds, BatchedEval* be, int P, int Dt, uint32_t max_nu,
-                 slc::SliceShape* sh) {
+                 const EvalConfig& ballot, slc::SliceShape* sh) {
   if (P < 16) return false;
   const int nb = slc::slice_bits(ds->rank_bytes, max_nu);
   int64_t tiles = 0;
@@ -574,12 +574,8 @@ bool level_slice(deoct_ctx* ctx, const deoct_dataset* ds, BatchedEval* be, int P
     e.ptile0 = tiles;
     tiles += slc::slice_tiles(e.count);
   }
-  // nodes of a few dozen samples leave most of a tile empty (n = 4000 over 64 nodes:
-  // 12.9 ms a fit against 11.9 with the re-laid kernel; n = 16000 over 32: 11.8 against 13.4)
-  int64_t samples = 0;
-  for (const EvalProb& e : be->probs) samples += e.count;
-  if (be->probs.size() > 1 && samples < 384 * tiles) return false;
-  if (!slc::slice_choose(ctx, Dt, ds->F, ds->K, P, nb, tiles, sh)) return false;
+  if (!slc::slice_choose(ctx, Dt, ds->F, ds->K, P, nb, tiles, (int)be->probs.size(), sh)) return false;
+  if (!slc::slice_wins(ctx, *sh, ballot)) return false;
   for (EvalProb& e : be->probs) {
     e.nb = nb;
     e.W = ds->rank_bytes;
@@ -725,7 +721,8 @@ int de_batched(deoct_ctx* ctx, const deoct_dataset* ds, const Compacted& c, uint
   }
   slc::SliceShape sh;
   // (an engine's launches run the ballot kernels, which read no planes)
-  const bool sliced = !ctx->engine && level_slice(ctx, ds, &be, P, Dt, max_nu, &sh);
+  const EvalConfig ballot = eval_choose_config(ctx, W, Dt, F, K, P, std::max<int64_t>(1, nsum_of(c, M)), M);
+  bool sliced = !ctx->engine && level_slice(ctx, ds, &be, P, Dt, max_nu, ballot, &sh);
   EvalConfig scfg;
   scfg.S = 1024;
   scfg.TG = sh.TG;
@@ -737,6 +734,7 @@ int de_batched(deoct_ctx* ctx, const deoct_dataset* ds, const Compacted& c, uint
     DEOCT_TRY(scratch_get(ctx, SL_EVAL_PROBS, sizeof(EvalProb) * M, (void**)&dep));
     DEOCT_TRY(build_plan(ctx, &be, scfg, F, K, P, s));
     level_planes(ctx, ds, &be, &sh);
+    if (sh.raw && !slice_once(ctx, nsum_of(c, M), P)) sliced = false;
   }
   DEOCT_TRY(upload(ctx, SL_EVAL_PROBS, be.probs, &dep, s));
   be.plan.d_probs = dep;
@@ -766,9 +764,8 @@ int de_batched(deoct_ctx* ctx, const deoct_dataset* ds, const Compacted& c, uint
   if (ctx->engine) {
     // S^1 and the first trials here, then the G generations in the engine's
     // launches shared with other jobs
-    EvalConfig cfg = eval_choose_config(ctx, W, Dt, F, K, P, std::max<int64_t>(1, nsum_of(c, M)), M);
-    DEOCT_TRY(build_plan(ctx, &be, cfg, F, K, P, s));
-    DEOCT_TRY(eval_launch(ctx, W, Dt, be.plan, cfg, s));
+    DEOCT_TRY(build_plan(ctx, &be, ballot, F, K, P, s));
+    DEOCT_TRY(eval_launch(ctx, W, Dt, be.plan, ballot, s));
     DEOCT_TRY(de_launch_step(ctx, a, 0, DE_FIRST | DE_GEN_DEVICE | (prm->gens >= 1 ? DE_TRIAL : 0), s));
     DEOCT_CUDA_TRY(cudaStreamSynchronize(s));
     if (prm->gens >= 1) DEOCT_TRY(engine_generations(ctx->engine, ctx, W, Dt, a, prm->gens, dp, be.probs));
@@ -779,7 +776,10 @@ int de_batched(deoct_ctx* ctx, const deoct_dataset* ds, const Compacted& c, uint
   int64_t nsum = 0;
   for (int m = 0; m < M; ++m) nsum += c.counts[m];
   const uint64_t key = tune_key(W, Dt, F, K, P, c.npad, M);
-  EvalConfig cfg = eval_choose_config(ctx, W, Dt, F, K, P, std::max<int64_t>(1, nsum / M), M);
+  // (the level's samples over its problems: a share of a share, as this was given before,
+  // chose shapes for smaller nodes; a level of 32 nodes of 1000 samples took 1.3 to 1.4 times
+  // as long a generation with them)
+  EvalConfig cfg = ballot;
   bool have = false;
   for (auto& kv : ctx->tuned)
     if (kv.first == key) {

@@ -37,6 +37,7 @@ EXPORTED = [
     "deoct_selftest_wait", "deoct_encode_auto", "deoct_engine_create", "deoct_engine_destroy",
     "deoct_engine_attach", "deoct_engine_get_stats", "deoct_get_memory", "deoct_fit_scratch_bound",
     "deoct_release_scratch", "deoct_set_scratch_limit", "deoct_set_eval_streaming", "deoct_get_slice_stats",
+    "deoct_set_eval_slicing",
 ]
 NOALLOC_SCRATCH_BYTES = 8 << 20
 
@@ -106,6 +107,7 @@ def load(path: str | None = None):
             "deoct_get_memory": [_vp, ctypes.POINTER(_u64), ctypes.POINTER(_u64)],
             "deoct_release_scratch": [_vp],
             "deoct_set_eval_streaming": [_vp, _i32],
+            "deoct_set_eval_slicing": [_vp, _i32],
             "deoct_set_scratch_limit": [_vp, _u64],
             "deoct_fit_scratch_bound": [_vp, _i64, _i32, _i32, _i32, ctypes.POINTER(Params),
                                         ctypes.POINTER(_u64)],
@@ -287,6 +289,11 @@ class Context:
     def set_eval_config(self, S=0, TG=0, warps=0, grid=0):
         """Force the evaluator's launch shape (0 = automatic); results are unchanged."""
         _check(load().deoct_set_eval_config(self.handle, S, TG, warps, grid))
+
+    def set_eval_slicing(self, mode: int):
+        """Evaluate with the bit-sliced kernel by the library's choice (0), wherever it can run (1)
+        or nowhere (-1); results unchanged."""
+        _check(load().deoct_set_eval_slicing(self.handle, int(mode)))
 
     def set_eval_streaming(self, on: bool):
         """Run every ballot-mode evaluation on the streaming kernel (results unchanged)."""

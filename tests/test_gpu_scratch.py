@@ -44,6 +44,8 @@ def _with(ds, fit, cap, forced, times=1):
     try:
         if forced:  # a forced launch shape keeps the fit off the bit-sliced evaluator and its planes
             ctx.set_eval_config(S=512, TG=32)
+        else:  # and this on it
+            ctx.set_eval_slicing(1)
         ctx.set_scratch_limit(cap)
         for _ in range(times):
             out = fit(ctx, ds)

@@ -1,5 +1,5 @@
-"""The bit-sliced evaluator through fits, which take it at any size, and through single
-evaluations large enough for it; every test asserts that it ran, and with how many digits a
+"""The bit-sliced evaluator through fits that are told to take it wherever it can run, and through
+single evaluations large enough for it; every test asserts that it ran, and with how many digits a
 threshold.  Ranks are drawn as such, with their n_p, so that small sets reach every digit
 count, with planes in memory and without ("raw": the context's scratch is capped at what the
 same fit holds on the other kernels, which leaves the planes no room)."""
@@ -48,6 +48,7 @@ def _fit(ds, prm, raw):
         else:  # as in a context that encoded the set: the planes' memory is there
             big = gpu_dataset(ctx, np.random.default_rng(0).random((20_000, 16)), np.zeros(20_000), 2, 2)
             del big
+        ctx.set_eval_slicing(1)
         ctx.reset_stats()
         pop = torch.empty((prm.pop, 2 * ((1 << prm.depth) - 1)), dtype=torch.float32, device="cuda")
         _, _, f = deoct.deoct_fit_subtree(ctx, ds, prm, pop_out=pop)
@@ -124,6 +125,7 @@ def test_contexts_fit_side_by_side():
     def work(job, times, out):
         X, y, K, prm = job
         ctx = deoct.Context(0)
+        ctx.set_eval_slicing(1)
         s = torch.cuda.Stream()
         with torch.cuda.stream(s):
             for _ in range(times):
