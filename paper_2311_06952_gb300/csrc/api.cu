@@ -412,8 +412,8 @@ int run_deoct(deoct_ctx* ctx, const deoct_dataset* ds, const int32_t* idx, int64
   };
   DEOCT_TRY(evaluate(s));
   // The generation number lives on the device (set to 1 by the init kernel and
-  // advanced by every trial step), so every generation is the same launches: captured
-  // as CUDA graphs and replayed.  With per-launch timing on, the launches are issued
+  // advanced by every trial step), so every generation is the same launches: built into
+  // CUDA graphs and replayed.  With per-launch timing on, the launches are issued
   // directly so that each evaluator launch gets its own events.
   DEOCT_TRY(de_launch_step(ctx, a, 0, DE_FIRST | DE_GEN_DEVICE | (p->gens >= 1 ? DE_TRIAL : 0), s));
   if (p->gens < 1) return DEOCT_OK;
@@ -426,55 +426,66 @@ int run_deoct(deoct_ctx* ctx, const deoct_dataset* ds, const int32_t* idx, int64
   }
   return replay_generations(
       ctx, p->gens,
-      [&](cudaStream_t st) {
-        DEOCT_TRY(evaluate(st));
-        return de_launch_step(ctx, a, 0, DE_SELECT | DE_TRIAL | DE_GEN_DEVICE, st);
+      [&] {
+        DEOCT_TRY(evaluate(s));
+        return de_launch_step(ctx, a, 0, DE_SELECT | DE_TRIAL | DE_GEN_DEVICE, s);
       },
       s);
 }
 
-// Generations captured in one graph: a generation of a small fit is about 10 us of two
+// Generations of one graph: a generation of a small fit is about 10 us of two
 // kernels, which a graph launch for each does not keep fed (n = 1000, 64 trees of depth
 // 2, G = 100: 1.29 ms with one generation a graph, 1.02 with eight).
 constexpr int kGensPerGraph = 8;
 
-int replay_generations(deoct_ctx* ctx, int G, const std::function<int(cudaStream_t)>& record, cudaStream_t s) {
-  if (!ctx->cap_stream)
-    DEOCT_CUDA_TRY(cudaStreamCreateWithFlags(&ctx->cap_stream, cudaStreamNonBlocking));
+int build_graph(deoct_ctx* ctx, const std::function<int()>& record, BuiltGraph* out) {
+  const uint64_t l0 = ctx->launches, e0 = ctx->eval_launches, s0 = ctx->slice_launches;
+  GraphBuild b;
+  DEOCT_CUDA_TRY(cudaGraphCreate(&b.graph, 0));
+  struct Building {  // ends with this scope, also by an exception
+    deoct_ctx* ctx;
+    cudaGraph_t graph;
+    ~Building() {
+      ctx->building = nullptr;
+      cudaGraphDestroy(graph);
+    }
+  } building{ctx, b.graph};
+  ctx->building = &b;
+  const int rc = record();
+  ctx->building = nullptr;
+  out->launches = ctx->launches - l0;
+  out->eval_launches = ctx->eval_launches - e0;
+  out->slice_launches = ctx->slice_launches - s0;
+  ctx->launches = l0;
+  ctx->eval_launches = e0;
+  ctx->slice_launches = s0;
+  DEOCT_TRY(rc);
+  out->exec = nullptr;
+  const cudaError_t ce = cudaGraphInstantiate(&out->exec, b.graph, 0);
+  if (ce != cudaSuccess) return set_error(DEOCT_ERR_CUDA, "graph instantiate failed: %s", cudaGetErrorString(ce));
+  return DEOCT_OK;
+}
+
+int replay_generations(deoct_ctx* ctx, int G, const std::function<int()>& record, cudaStream_t s) {
   for (const int gens : {std::min(G, kGensPerGraph), G % std::min(G, kGensPerGraph)}) {
     if (gens == 0) break;
     const int replays = gens == std::min(G, kGensPerGraph) ? G / gens : 1;
-    const uint64_t l0 = ctx->launches, e0 = ctx->eval_launches, s0 = ctx->slice_launches;
-    cudaGraph_t graph = nullptr;
-    cudaGraphExec_t exec = nullptr;
-    DEOCT_CUDA_TRY(cudaStreamBeginCapture(ctx->cap_stream, cudaStreamCaptureModeThreadLocal));
-    int rc = DEOCT_OK;
-    for (int i = 0; i < gens && rc == DEOCT_OK; ++i) rc = record(ctx->cap_stream);
-    cudaError_t ce = cudaStreamEndCapture(ctx->cap_stream, &graph);
-    const uint64_t per_launch = ctx->launches - l0, per_eval = ctx->eval_launches - e0;
-    const uint64_t per_slice = ctx->slice_launches - s0;
-    ctx->launches = l0;
-    ctx->eval_launches = e0;
-    ctx->slice_launches = s0;
-    if (rc != DEOCT_OK) {
-      if (graph) cudaGraphDestroy(graph);
-      return rc;
-    }
-    if (ce != cudaSuccess) return set_error(DEOCT_ERR_CUDA, "graph capture failed: %s", cudaGetErrorString(ce));
-    ce = cudaGraphInstantiate(&exec, graph, 0);
-    if (ce != cudaSuccess) {
-      cudaGraphDestroy(graph);
-      return set_error(DEOCT_ERR_CUDA, "graph instantiate failed: %s", cudaGetErrorString(ce));
-    }
+    BuiltGraph g;
+    DEOCT_TRY(build_graph(
+        ctx,
+        [&] {
+          for (int i = 0; i < gens; ++i) DEOCT_TRY(record());
+          return (int)DEOCT_OK;
+        },
+        &g));
+    cudaError_t ce = cudaSuccess;
     for (int r = 0; r < replays && ce == cudaSuccess; ++r) {
-      ce = cudaGraphLaunch(exec, s);
-      ctx->launches += per_launch;
-      ctx->eval_launches += per_eval;
-      ctx->slice_launches += per_slice;
+      ce = cudaGraphLaunch(g.exec, s);
+      ctx->launches += g.launches;
+      ctx->eval_launches += g.eval_launches;
+      ctx->slice_launches += g.slice_launches;
     }
-    // the graph may be destroyed once its launches are queued
-    cudaGraphExecDestroy(exec);
-    cudaGraphDestroy(graph);
+    cudaGraphExecDestroy(g.exec);  // (may be destroyed once its launches are queued)
     if (ce != cudaSuccess) return set_error(DEOCT_ERR_CUDA, "graph launch failed: %s", cudaGetErrorString(ce));
   }
   return DEOCT_OK;
@@ -545,7 +556,6 @@ int deoct_destroy(deoct_ctx* ctx) {
   for (int i = 0; i < SL_COUNT; ++i)
     if (ctx->scratch[i].ptr) cudaFree(ctx->scratch[i].ptr);
   if (ctx->d_status) cudaFree(ctx->d_status);
-  if (ctx->cap_stream) cudaStreamDestroy(ctx->cap_stream);
   if (ctx->h_pinned) cudaFreeHost(ctx->h_pinned);
   for (cudaEvent_t ev : ctx->ev_pairs) cudaEventDestroy(ev);
   delete ctx;

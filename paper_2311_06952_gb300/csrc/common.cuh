@@ -9,6 +9,8 @@
 #include <cstdio>
 #include <array>
 #include <string>
+#include <tuple>
+#include <type_traits>
 #include <vector>
 
 #include "../../include/deoct.h"
@@ -78,6 +80,12 @@ enum ScratchSlot : int {
   SL_COUNT
 };
 
+// A chain of kernel nodes under construction (build_graph).
+struct GraphBuild {
+  cudaGraph_t graph = nullptr;
+  cudaGraphNode_t last = nullptr;
+};
+
 struct deoct_ctx_impl;
 
 }  // namespace deoct
@@ -87,7 +95,7 @@ struct deoct_ctx {
   int num_sms = 0;
   int max_smem_optin = 0;
   int smem_per_sm = 0;
-  cudaStream_t cap_stream = nullptr;  // private stream used only to capture CUDA graphs
+  deoct::GraphBuild* building = nullptr;  // the graph that launch_kernel adds to instead of launching
   int* d_status = nullptr;  // device status word (bits ST_*)
   deoct::Scratch scratch[deoct::SL_COUNT];
   // pinned host staging for small read-backs
@@ -135,6 +143,41 @@ int check_status(deoct_ctx* ctx, cudaStream_t stream);
 // launch accounting
 inline void count_launch(deoct_ctx* ctx, int n = 1) { ctx->launches += (uint64_t)n; }
 int check_launch(const char* what);
+
+// Launch a kernel on s, or add it to the graph the context is building: the launches of a
+// generation, which are replayed.  Graphs are built of nodes and not captured from a
+// stream: a capture, whatever its mode, is ended by any other thread that synchronises
+// the device, and on this driver that thread can crash.
+template <typename... P, typename... A>
+inline int launch_on(deoct_ctx* ctx, const char* what, void (*kern)(P...), int grid, int block, size_t smem,
+                     cudaStream_t s, const A&... args) {
+  std::tuple<std::decay_t<P>...> vals(args...);
+  const cudaError_t e = std::apply(
+      [&](auto&... v) {
+        void* ptr[] = {static_cast<void*>(&v)...};
+        if (!ctx->building)
+          return cudaLaunchKernel(reinterpret_cast<const void*>(kern), dim3((unsigned)grid), dim3((unsigned)block), ptr,
+                                  smem, s);
+        GraphBuild& b = *ctx->building;
+        cudaKernelNodeParams np = {};
+        np.func = reinterpret_cast<void*>(kern);
+        np.gridDim = dim3((unsigned)grid);
+        np.blockDim = dim3((unsigned)block);
+        np.sharedMemBytes = (unsigned)smem;
+        np.kernelParams = ptr;  // (copied)
+        cudaGraphNode_t node = nullptr;
+        const cudaError_t r = cudaGraphAddKernelNode(&node, b.graph, &b.last, b.last ? 1 : 0, &np);
+        if (r == cudaSuccess) b.last = node;
+        return r;
+      },
+      vals);
+  if (e != cudaSuccess) {
+    cudaGetLastError();
+    return set_error(DEOCT_ERR_CUDA, "launch of %s failed: %s", what, cudaGetErrorString(e));
+  }
+  count_launch(ctx);
+  return DEOCT_OK;
+}
 int validate_dataset(const deoct_dataset* ds);
 
 // Set a kernel's dynamic shared-memory limit to the largest value the device

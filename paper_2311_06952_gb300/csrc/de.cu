@@ -661,22 +661,15 @@ int de_launch_step(deoct_ctx* ctx, const DEArgs& a, int g, int flags, cudaStream
     int lg = 0;  // lanes an individual (log2)
     while (lg < kStepLanes && (2 << lg) <= (1 << a.depth) && (a.P << lg) * 2 <= 1024) ++lg;
     DEOCT_TRY(set_max_dynamic_smem(ctx, de_step_chip_kernel));
-    de_step_chip_kernel<<<nprob, block_for(a.P << lg), smem, s>>>(a, g, flags, lg);
-    count_launch(ctx);
-    return check_launch("de_step_chip_kernel");
+    return launch_on(ctx, "de_step_chip_kernel", de_step_chip_kernel, nprob, block_for(a.P << lg), smem, s, a, g, flags,
+                     lg);
   }
   if (steady && !a.probs && a.part_f && a.P > kStepP && a.P <= kMaxPop) {
     const int nblk = (a.P + kDeWideR - 1) / kDeWideR;
-    de_select_wide_kernel<<<nblk, kDeWideR * kDeWideG, 0, s>>>(a, g, flags);
-    count_launch(ctx);
-    DEOCT_TRY(check_launch("de_select_wide_kernel"));
-    de_trial_wide_kernel<<<nblk, kDeWideR * kDeWideG, 0, s>>>(a, flags, nblk);
-    count_launch(ctx);
-    return check_launch("de_trial_wide_kernel");
+    DEOCT_TRY(launch_on(ctx, "de_select_wide_kernel", de_select_wide_kernel, nblk, kDeWideR * kDeWideG, 0, s, a, g, flags));
+    return launch_on(ctx, "de_trial_wide_kernel", de_trial_wide_kernel, nblk, kDeWideR * kDeWideG, 0, s, a, flags, nblk);
   }
-  de_step_kernel<<<nprob, block_for(a.P * lanes), 0, s>>>(a, g, flags, lanes);
-  count_launch(ctx);
-  return check_launch("de_step_kernel");
+  return launch_on(ctx, "de_step_kernel", de_step_kernel, nprob, block_for(a.P * lanes), 0, s, a, g, flags, lanes);
 }
 
 int launch_best_extract(deoct_ctx* ctx, const float* pop, const double* fit, const int32_t* best,

@@ -12,7 +12,7 @@
 // so that a small job does not tick at the pace of a large one.  One tick of a
 // group is one evaluator launch over every problem's trials and one DE-step
 // launch (Eq. selection, best, next trials of Algorithm 4).  Each group has its
-// own stream and replays its captured tick as long as its set of problems does
+// own stream and replays its tick's graph as long as its set of problems does
 // not change; the GPU overlaps the groups' streams.  Each problem keeps its own
 // data, Philox key (seed, node id) and device-side generation counter, so
 // problems join at any tick and leave after exactly their G generations: a
@@ -83,7 +83,7 @@ struct EngineSub {
 
 namespace {
 
-// One group of the active set: its problems, stream, captured tick and device
+// One group of the active set: its problems, stream, tick graph and device
 // arrays.
 struct Group {
   std::vector<EngineSub*> subs;
@@ -104,7 +104,7 @@ struct Group {
 
 struct deoct_engine {
   int device = 0;
-  deoct_ctx* ctx = nullptr;  // the engine's own context: status word, counters, capture stream
+  deoct_ctx* ctx = nullptr;  // the engine's own context: status word and counters
   std::thread thr;
   std::mutex mu;
   std::condition_variable cv;
@@ -171,7 +171,7 @@ int engine_upload(deoct_engine* e, cudaStream_t s, const std::vector<T>& h, T** 
   return DEOCT_OK;
 }
 
-// Upload the arrays of group g's problems and capture its tick (evaluator + DE
+// Upload the arrays of group g's problems and build its tick (evaluator + DE
 // step) as a graph.
 int rebuild(deoct_engine* e, const EngineGroupKey& k, Group& g) {
   if (g.exec) {
@@ -237,28 +237,17 @@ int rebuild(deoct_engine* e, const EngineGroupKey& k, Group& g) {
   a.dither = k.dither;
   a.Kmax = Kmax;
   a.status = c->d_status;
-  if (!c->cap_stream) DEOCT_CUDA_TRY(cudaStreamCreateWithFlags(&c->cap_stream, cudaStreamNonBlocking));
-  const uint64_t l0 = c->launches, v0 = c->eval_launches;
-  cudaGraph_t graph = nullptr;
-  DEOCT_CUDA_TRY(cudaStreamBeginCapture(c->cap_stream, cudaStreamCaptureModeThreadLocal));
-  int rc = eval_launch(c, k.W, k.Dt, plan, cfg, c->cap_stream);
-  if (rc == DEOCT_OK) rc = de_launch_step(c, a, 0, DE_SELECT | DE_TRIAL | DE_GEN_DEVICE, c->cap_stream);
-  cudaError_t ce = cudaStreamEndCapture(c->cap_stream, &graph);
-  g.per_replay_launches = c->launches - l0;
-  g.per_replay_evals = c->eval_launches - v0;
-  c->launches = l0;
-  c->eval_launches = v0;
-  if (rc != DEOCT_OK) {
-    if (graph) cudaGraphDestroy(graph);
-    return rc;
-  }
-  if (ce != cudaSuccess) return set_error(DEOCT_ERR_CUDA, "engine graph capture failed: %s", cudaGetErrorString(ce));
-  ce = cudaGraphInstantiate(&g.exec, graph, 0);
-  cudaGraphDestroy(graph);
-  if (ce != cudaSuccess) {
-    g.exec = nullptr;
-    return set_error(DEOCT_ERR_CUDA, "engine graph instantiate failed: %s", cudaGetErrorString(ce));
-  }
+  BuiltGraph tick;
+  DEOCT_TRY(build_graph(
+      c,
+      [&] {
+        DEOCT_TRY(eval_launch(c, k.W, k.Dt, plan, cfg, g.stream));
+        return de_launch_step(c, a, 0, DE_SELECT | DE_TRIAL | DE_GEN_DEVICE, g.stream);
+      },
+      &tick));
+  g.exec = tick.exec;
+  g.per_replay_launches = tick.launches;
+  g.per_replay_evals = tick.eval_launches;
   g.dirty = false;
   return DEOCT_OK;
 }

@@ -622,7 +622,7 @@ int eval_launch(deoct_ctx* ctx, int W, int D, const EvalPlan& plan, const EvalCo
   cudaEvent_t e0 = nullptr, e1 = nullptr;
   cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
   DEOCT_CUDA_TRY(cudaStreamIsCapturing(stream, &cs));
-  const bool timed = ctx->timing && cs == cudaStreamCaptureStatusNone;  // not inside graphs
+  const bool timed = ctx->timing && !ctx->building && cs == cudaStreamCaptureStatusNone;  // not inside graphs
   if (timed) {
     DEOCT_CUDA_TRY(cudaEventCreate(&e0));
     DEOCT_CUDA_TRY(cudaEventCreate(&e1));

@@ -782,9 +782,7 @@ int launch_kernel(deoct_ctx* ctx, Kern kern, const EvalArgs& args, const EvalCon
   }
   if ((int64_t)grid > args.total_tiles) grid = (int)args.total_tiles;
   if (grid < 1) return DEOCT_OK;
-  kern<<<grid, cfg.warps * 32, smem, s>>>(args);
-  count_launch(ctx);
-  return check_launch(name);
+  return launch_on(ctx, name, kern, grid, cfg.warps * 32, smem, s, args);
 }
 
 // eval_stream.cu: the streaming kernel for uint16 (W = 2) or uint32 (W = 4)

@@ -201,7 +201,7 @@ int slice_launch(deoct_ctx* ctx, int D, const EvalPlan& plan, const SliceShape& 
   cudaEvent_t e0 = nullptr, e1 = nullptr;
   cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
   DEOCT_CUDA_TRY(cudaStreamIsCapturing(s, &cs));
-  const bool timed = ctx->timing && cs == cudaStreamCaptureStatusNone;  // not inside graphs
+  const bool timed = ctx->timing && !ctx->building && cs == cudaStreamCaptureStatusNone;  // not inside graphs
   if (timed) {
     DEOCT_CUDA_TRY(cudaEventCreate(&e0));
     DEOCT_CUDA_TRY(cudaEventCreate(&e1));

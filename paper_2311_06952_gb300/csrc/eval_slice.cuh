@@ -863,9 +863,7 @@ template <int D, int ND>
 int launch_slice_t(deoct_ctx* ctx, const SliceArgs& sa, bool raw, int grid, cudaStream_t s) {
   auto* kern = raw ? eval_slice_kernel<D, ND, true> : eval_slice_kernel<D, ND, false>;
   DEOCT_TRY(set_max_dynamic_smem(ctx, kern));
-  kern<<<grid, kWarps * 32, (size_t)sa.smem_bytes, s>>>(sa);
-  count_launch(ctx);
-  return check_launch("eval_slice_kernel");
+  return launch_on(ctx, "eval_slice_kernel", kern, grid, kWarps * 32, (size_t)sa.smem_bytes, s, sa);
 }
 template <int D>
 int launch_slice_d(deoct_ctx* ctx, int nd, const SliceArgs& sa, bool raw, int grid, cudaStream_t s) {

@@ -237,10 +237,16 @@ int radix_sort_segments(deoct_ctx* ctx, uint32_t* k0, uint32_t* v0, uint32_t* k1
 int engine_generations(deoct_engine* e, const void* owner, int W, int Dt, const DEArgs& a, int G,
                        const std::vector<DEProb>& dp, const std::vector<EvalProb>& ep);
 
-// G generations, each the launches `record` issues on the stream it is given, on
-// stream s: kGensPerGraph of them captured as one graph and replayed, the remainder
-// as another (api.cu).  The graphs may be destroyed once this returns.
-int replay_generations(deoct_ctx* ctx, int G, const std::function<int(cudaStream_t)>& record, cudaStream_t s);
+// The launches `record` issues (launch_on), one after another as a graph, which the caller
+// destroys (api.cu); the context's counters are left as they were.
+struct BuiltGraph {
+  cudaGraphExec_t exec = nullptr;
+  uint64_t launches = 0, eval_launches = 0, slice_launches = 0;
+};
+int build_graph(deoct_ctx* ctx, const std::function<int()>& record, BuiltGraph* out);
+// G generations, each the launches `record` issues, on stream s: kGensPerGraph of them
+// built into one graph and replayed, the remainder as another (api.cu).
+int replay_generations(deoct_ctx* ctx, int G, const std::function<int()>& record, cudaStream_t s);
 // the columns of a (sub)set ordered by class (mh.cu); tmp: 3072 bytes of device memory
 int class_order(deoct_ctx* ctx, const deoct_dataset* ds, const int32_t* idx, int64_t n, int32_t* order, void* tmp,
                 cudaStream_t s);

@@ -11,7 +11,7 @@
 //   D_t >= 2: DEOCT of depth D_t (Philox stream = node id), either
 //     - plain: one DEOCT per node, each with its own launches, or
 //     - batched: one multi-problem evaluator launch and one DE-step launch per
-//       generation for all nodes of the level, replayed from captured CUDA graphs
+//       generation for all nodes of the level, replayed from CUDA graphs
 //       of eight generations: the bit-sliced evaluator over the level's bit planes
 //       (level_planes), or the ballot kernels with a shape an autotuner picks;
 //   D_t = 1: exhaustive depth-1 search: per feature, the (node, rank) keys of
@@ -659,7 +659,7 @@ uint64_t tune_key(int W, int D, int F, int K, int P, int64_t npad, int M) {
 }
 
 // Batched DEOCT for all segments of a level: one evaluator launch and one DE
-// step launch per generation, replayed from a captured CUDA graph.
+// step launch per generation, replayed from a CUDA graph.
 int de_batched(deoct_ctx* ctx, const deoct_dataset* ds, const Compacted& c, uint32_t max_nu,
                const std::vector<int>& node_ids, int Dt, const deoct_params* prm,
                const float* d_seeds, int S, std::vector<uint16_t>* ra, std::vector<uint32_t>* rth,
@@ -891,15 +891,15 @@ int de_batched(deoct_ctx* ctx, const deoct_dataset* ds, const Compacted& c, uint
   if (sliced) cfg = scfg;
   else DEOCT_TRY(build_plan(ctx, &be, cfg, F, K, P, s));
 
-  // ---- S^1, then G generations from captured graphs --------------------------
+  // ---- S^1, then G generations from graphs ------------------------------------
   DEOCT_TRY(evaluate(cfg, s));
   DEOCT_TRY(de_launch_step(ctx, a, 0, DE_FIRST | DE_GEN_DEVICE | (prm->gens >= 1 ? DE_TRIAL : 0), s));
   if (prm->gens >= 1) {
     DEOCT_TRY(replay_generations(
         ctx, prm->gens,
-        [&](cudaStream_t st) {
-          DEOCT_TRY(evaluate(cfg, st));
-          return de_launch_step(ctx, a, 0, DE_SELECT | DE_TRIAL | DE_GEN_DEVICE, st);
+        [&] {
+          DEOCT_TRY(evaluate(cfg, s));
+          return de_launch_step(ctx, a, 0, DE_SELECT | DE_TRIAL | DE_GEN_DEVICE, s);
         },
         s));
     const cudaError_t ce = cudaStreamSynchronize(s);
