@@ -199,7 +199,7 @@ static bool slice_plan(const deoct_ctx* ctx, const deoct_dataset* ds, const int3
                        int depth, int64_t max_nu, EvalPlan* plan, slc::SliceShape* sh) {
   if (n_sub < 1 || P < 16) return false;  // (fewer trees run on the streaming kernel)
   const int W = ds->rank_bytes, nb = slc::slice_bits(W, (uint32_t)max_nu);
-  if (!slc::slice_choose(ctx, depth, ds->F, ds->K, P, nb, slc::slice_tiles(n_sub), 0, sh)) return false;
+  if (!slc::slice_choose(ctx, W, rows_copied(ds, idx), depth, ds->F, ds->K, P, nb, slc::slice_tiles(n_sub), 0, sh)) return false;
   EvalConfig cfg;
   cfg.S = 1024;
   cfg.TG = sh->TG;
@@ -236,27 +236,31 @@ static int slice_planes_of_fit(deoct_ctx* ctx, const deoct_dataset* ds, const in
   return slc::slice_planes(ctx, ds->rank_bytes, *plan, nullptr, 1, tiles, s);
 }
 
-// One evaluation on its own: whether the bit-sliced evaluator, which then transposes
-// every tile's ranks itself, is the faster one (GB300: 100 to 128 trees 150 us against
-// 145 at n = 1e6, F = 30, depth 3, 49 against 45 at n = 2e5, K = 10; 256 trees 39
-// against 35 us at n = 1e5, F = 20, depth 3, 500 against 790 at n = 2e6, depth 5; 1024
-// trees 4.5 ms against 10.2 at n = 1e7, depth 4).
-bool slice_once(const deoct_ctx* ctx, int64_t n_sub, int P) {
-  return ctx->force_slice > 0 || (P >= 192 && n_sub * P >= (int64_t(1) << 27));
-}
-
 // Bound of an encoded set's ranks that needs no look at the device: its size, and
 // the rank width.  (Where a set breaks it the evaluator still counts right, slowly.)
 static int64_t width_bound(const deoct_dataset* ds) { return std::min<int64_t>(ds->n, ds->rank_bytes == 2 ? 65536 : kMaxN); }
 
-// evaluate one population on one (sub)set with the re-laid or the streaming kernel:
-// counts must be zero beforehand
+// the ballot kernels' shape for one population on one (sub)set
+static EvalConfig ballot_config(deoct_ctx* ctx, const deoct_dataset* ds, const int32_t* idx, int64_t n_sub, int P,
+                                int depth) {
+  return eval_choose_config(ctx, ds->rank_bytes, depth, ds->F, ds->K, P, std::max<int64_t>(1, n_sub), 1,
+                            rows_copied(ds, idx));
+}
+
+// evaluate one population on one (sub)set with them: counts must be zero beforehand
 static int eval_ballot(deoct_ctx* ctx, const deoct_dataset* ds, const int32_t* idx, int64_t n_sub,
-                       const uint32_t* nodes, uint32_t* counts, int P, int depth, cudaStream_t s) {
+                       const uint32_t* nodes, uint32_t* counts, int P, int depth, const EvalConfig& cfg,
+                       cudaStream_t s) {
   if (n_sub == 0) return DEOCT_OK;
-  EvalConfig cfg = eval_choose_config(ctx, ds->rank_bytes, depth, ds->F, ds->K, P, n_sub, 1, rows_copied(ds, idx));
   EvalPlan plan = single_eval_plan(ds, idx, n_sub, nodes, counts, P, cfg);
   return eval_launch(ctx, ds->rank_bytes, depth, plan, cfg, s);
+}
+
+// whether one evaluation on its own takes the bit-sliced evaluator, with its plan and shape
+static bool once_sliced(const deoct_ctx* ctx, const deoct_dataset* ds, const int32_t* idx, int64_t n_sub, int P, int depth,
+                        const EvalConfig& ballot, EvalPlan* plan, slc::SliceShape* sh) {
+  return slc::slice_once(ctx, n_sub, P) && slice_plan(ctx, ds, idx, n_sub, P, depth, width_bound(ds), plan, sh) &&
+         slc::slice_wins_once(ctx, *sh, ballot);
 }
 
 // the same with the evaluator that suits the shape
@@ -264,14 +268,15 @@ static int eval_single(deoct_ctx* ctx, const deoct_dataset* ds, const int32_t* i
                        const uint32_t* nodes, uint32_t* counts, int P, int depth,
                        cudaStream_t s) {
   if (n_sub == 0) return DEOCT_OK;
+  const EvalConfig ballot = ballot_config(ctx, ds, idx, n_sub, P, depth);
   EvalPlan sp;
   slc::SliceShape sh;
-  if (slice_once(ctx, n_sub, P) && slice_plan(ctx, ds, idx, n_sub, P, depth, width_bound(ds), &sp, &sh)) {
+  if (once_sliced(ctx, ds, idx, n_sub, P, depth, ballot, &sp, &sh)) {
     sp.single.nodes = nodes;
     sp.single.counts = counts;
     return slc::slice_launch(ctx, depth, sp, sh, s);
   }
-  return eval_ballot(ctx, ds, idx, n_sub, nodes, counts, P, depth, s);
+  return eval_ballot(ctx, ds, idx, n_sub, nodes, counts, P, depth, ballot, s);
 }
 
 // One evaluation of caller-given trees in a single launch: the evaluator packs
@@ -288,9 +293,10 @@ static int eval_single_fused(deoct_ctx* ctx, const deoct_dataset* ds, const int3
   uint32_t* base = nullptr;
   DEOCT_TRY(scratch_get(ctx, SL_EVAL_ACC, bytes, (void**)&base));
   if (grows) DEOCT_CUDA_TRY(cudaMemsetAsync(base, 0, ctx->scratch[SL_EVAL_ACC].bytes, s));
+  const EvalConfig cfg = ballot_config(ctx, ds, idx, n_sub, P, depth);
   EvalPlan sp;
   slc::SliceShape sh;
-  if (slice_once(ctx, n_sub, P) && slice_plan(ctx, ds, idx, n_sub, P, depth, width_bound(ds), &sp, &sh)) {
+  if (once_sliced(ctx, ds, idx, n_sub, P, depth, cfg, &sp, &sh)) {
     sp.single.a16 = a;
     sp.single.th32 = theta;
     sp.single.counts = base + 4;
@@ -299,7 +305,6 @@ static int eval_single_fused(deoct_ctx* ctx, const deoct_dataset* ds, const int3
     sp.errors_out = errors_out;
     return slc::slice_launch(ctx, depth, sp, sh, s);
   }
-  EvalConfig cfg = eval_choose_config(ctx, ds->rank_bytes, depth, ds->F, ds->K, P, n_sub, 1, rows_copied(ds, idx));
   EvalPlan plan = single_eval_plan(ds, idx, n_sub, nullptr, base + 4, P, cfg);
   plan.single.a16 = a;
   plan.single.th32 = theta;
@@ -383,8 +388,7 @@ int run_deoct(deoct_ctx* ctx, const deoct_dataset* ds, const int32_t* idx, int64
   slc::SliceShape sh;
   // the ballot kernels' modelled time; n_p is read back, which waits for the stream, only
   // where the bit-sliced evaluator would win with one bit a rank
-  const EvalConfig ballot = eval_choose_config(ctx, ds->rank_bytes, p->depth, ds->F, ds->K, p->pop,
-                                               std::max<int64_t>(1, n_sub), 1, rows_copied(ds, idx));
+  const EvalConfig ballot = ballot_config(ctx, ds, idx, n_sub, p->pop, p->depth);
   auto wins = [&](int64_t nu) {
     return slice_plan(ctx, ds, idx, n_sub, p->pop, p->depth, nu, &sp, &sh) && slc::slice_wins(ctx, sh, ballot);
   };
@@ -404,11 +408,11 @@ int run_deoct(deoct_ctx* ctx, const deoct_dataset* ds, const int32_t* idx, int64
     if (p->gens >= 1) DEOCT_TRY(slice_planes_of_fit(ctx, ds, idx, n_sub, &sp, s));
     sh.raw = sp.single.planes == nullptr;
     // without planes every generation transposes the ranks again, as one evaluation does
-    if (sh.raw && !slice_once(ctx, n_sub, p->pop)) sliced = false;
+    if (sh.raw && !(slc::slice_once(ctx, n_sub, p->pop) && slc::slice_wins_once(ctx, sh, ballot))) sliced = false;
   }
   auto evaluate = [&](cudaStream_t st) {
     return sliced ? slc::slice_launch(ctx, p->depth, sp, sh, st)
-                  : eval_ballot(ctx, ds, idx, n_sub, b.nodes, b.counts, p->pop, p->depth, st);
+                  : eval_ballot(ctx, ds, idx, n_sub, b.nodes, b.counts, p->pop, p->depth, ballot, st);
   };
   DEOCT_TRY(evaluate(s));
   // The generation number lives on the device (set to 1 by the init kernel and

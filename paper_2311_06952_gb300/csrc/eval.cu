@@ -419,7 +419,7 @@ EvalConfig eval_choose_config(deoct_ctx* ctx, int W, int D, int F, int K, int P,
       // sweeps at n = 1e5, F = 20 and n = 1e7, F = 10.  Few large items leave
       // CTAs idle in the last wave; many small ones pay the overhead.
       const int64_t ncta = 2 * (int64_t)ctx->num_sms;
-      double best = -1.0;
+      double best = -1.0, best_waves = 0.0;
       for (int S : {2048, 1024, 512, 256})
         for (int TG : {256, 128, 64, 32, 16}) {
           const int tg = std::min(TG, P);
@@ -430,6 +430,7 @@ EvalConfig eval_choose_config(deoct_ctx* ctx, int W, int D, int F, int K, int P,
           const double cost = waves * ((double)S * tg + 7000.0 + 170.0 * copies);
           if (best < 0 || cost < best) {
             best = cost;
+            best_waves = 2.0 * waves;
             c.S = S;
             c.TG = tg;
           }
@@ -451,15 +452,17 @@ EvalConfig eval_choose_config(deoct_ctx* ctx, int W, int D, int F, int K, int P,
           const double cost = waves * ((double)S * tg + 25000.0 + 170.0 * copies) / 2.13;
           if (best < 0 || cost < best) {
             best = cost;
+            best_waves = waves;
             c.S = S;
             c.TG = tg;
             c.warps = 32;
           }
         }
       // time of a launch in us, fitted to 649 random shapes (see slice_choose; standard
-      // deviation 11%)
+      // deviation 11%), and what gathering the rows adds to it (36 shapes)
       const int Q = bins_per_lane(D, (1 << D) * K);
-      c.us = best < 0 ? 1e30 : 5.45 + 0.81 * (5 - D) + best * (9.08e-5 * D + 2.43e-5 * (Q - 1));
+      c.us = best < 0 ? 1e30 : 5.45 + 0.81 * (5 - D) + best * (9.08e-5 * D + 2.43e-5 * (Q - 1)) +
+                                   (copied ? 0.0 : 4.0e-4 * best_waves * c.S * F);
       if (best < 0) {  // nothing keeps two CTAs per SM: the largest shape that fits
         c.S = 2048;
         c.TG = std::min(P, 256);

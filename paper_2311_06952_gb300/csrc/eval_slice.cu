@@ -82,7 +82,8 @@ int slice_bits(int W, uint32_t max_nu) {
   return b;
 }
 
-bool slice_choose(const deoct_ctx* ctx, int D, int F, int K, int P, int nb, int64_t tiles, int nprob, SliceShape* out) {
+bool slice_choose(const deoct_ctx* ctx, int W, bool copied, int D, int F, int K, int P, int nb, int64_t tiles, int nprob,
+                  SliceShape* out) {
   if (D < 1 || D > kMaxDepthSlice || P < 1 || tiles < 1) return false;
   if (ctx->force_S || ctx->force_TG || ctx->force_warps || ctx->force_grid || ctx->force_stream || ctx->force_slice < 0)
     return false;
@@ -137,6 +138,11 @@ bool slice_choose(const deoct_ctx* ctx, int D, int F, int K, int P, int nb, int6
   out->us = 7.28 + 0.0038 * F * nd +
             waves * (0.595 + 8.2e-4 * F * (digit_rows(nb, nd) + nb) + loads * (0.00996 * rounds + 0.0015 * quads) +
                      0.2845 * rounds * leaves8 * classes);
+  // The same without planes, fitted to 236 random shapes of 2^27 tree-samples and more
+  // (192 to 4096 trees; standard deviation 12%): ranks and class rows are transposed in
+  // the launch, and every tile holds every class.
+  out->us_raw = 25.25 + waves * (loads * (0.0207 * rounds + 0.00107 * quads) + 0.161 * rounds * leaves8 * K +
+                                 F * ((W == 2 ? 0.072 : 0.148) + (copied ? 0.0 : 0.49)) + 1.08 * K);
   return true;
 }
 
@@ -150,6 +156,21 @@ bool slice_choose(const deoct_ctx* ctx, int D, int F, int K, int P, int nb, int6
 // 512 trees of depth 4 181 / 64.
 bool slice_wins(const deoct_ctx* ctx, const SliceShape& s, const EvalConfig& ballot) {
   return ctx->force_slice > 0 || s.us < 1.05 * ballot.us;
+}
+
+// One evaluation on its own, whose tiles' ranks the kernel transposes itself.  Below 192
+// trees or 2^27 tree-samples the ballot kernels were level or ahead (GB300: 100 to 128 trees
+// 150 us bit-sliced against 145 at n = 1e6, F = 30, depth 3, 49 against 45 at n = 2e5, K = 10;
+// 256 trees 39 against 35 at n = 1e5, F = 20, depth 3).  Above, by the models: of 236 random
+// shapes the bit-sliced one was the slower at 53 (1201 trees of depth 5, n = 1.35e6, F = 30,
+// uint32 7.16 ms against 3.10; 931, n = 1.5e5, K = 9 814 us against 381), taken by them 4,
+// by 7% at most; 256 trees of depth 5 on 2e6 rows 500 us against 790, 1024 of depth 4 on 1e7
+// 4.5 ms against 10.2.
+bool slice_once(const deoct_ctx* ctx, int64_t n, int P) {
+  return ctx->force_slice > 0 || (P >= 192 && n * P >= (int64_t(1) << 27));
+}
+bool slice_wins_once(const deoct_ctx* ctx, const SliceShape& s, const EvalConfig& ballot) {
+  return ctx->force_slice > 0 || s.us_raw < 0.95 * ballot.us;
 }
 
 int slice_planes(deoct_ctx* ctx, int W, const EvalPlan& plan, const EvalProb* d_probs, int nprob, int64_t tiles,

@@ -89,16 +89,22 @@ namespace slc {
 struct SliceShape {
   int TG = 0, nd = 0, rows = 0, rec_bytes = 0;
   bool raw = true;  // no planes in memory (all of a launch's problems have them, or none)
-  double us = 0;    // modelled time of a launch with planes
+  double us = 0, us_raw = 0;  // modelled time of a launch with planes, and without
 };
 int64_t slice_tiles(int64_t count);                // tiles of 1024 samples
 size_t slice_plane_bytes(int64_t tiles, int F, int K, int nb);
 int slice_bits(int W, uint32_t max_nu);            // planes that hold every theta < max_nu
 // nb: planes per feature; tiles: of all problems, for one tree group; nprob: problems
 // whose samples are ordered by class (0: one, ordered only with 2 K tiles or more)
-bool slice_choose(const deoct_ctx* ctx, int D, int F, int K, int P, int nb, int64_t tiles, int nprob, SliceShape* out);
+// W, copied: rank width and whether the rows are copied or gathered (launches without planes)
+bool slice_choose(const deoct_ctx* ctx, int W, bool copied, int D, int F, int K, int P, int nb, int64_t tiles, int nprob,
+                  SliceShape* out);
 // Whether the generations of a fit are faster on it than on the ballot kernels.
 bool slice_wins(const deoct_ctx* ctx, const SliceShape& s, const EvalConfig& ballot);
+// The same for an evaluation without planes: whether `n` samples are a case for it, and its
+// shape the faster one.
+bool slice_once(const deoct_ctx* ctx, int64_t n, int P);
+bool slice_wins_once(const deoct_ctx* ctx, const SliceShape& s, const EvalConfig& ballot);
 int slice_planes(deoct_ctx* ctx, int W, const EvalPlan& plan, const EvalProb* d_probs, int nprob, int64_t tiles,
                  cudaStream_t s);
 int slice_launch(deoct_ctx* ctx, int D, const EvalPlan& plan, const SliceShape& shape, cudaStream_t s);
@@ -133,8 +139,6 @@ void eval_build_jobs(const std::vector<int64_t>& counts, const std::vector<int>&
 int launch_errors(deoct_ctx* ctx, const uint32_t* counts, int P, int L, int K, int64_t n_valid,
                   uint32_t* errors, cudaStream_t stream, const int* status = nullptr);
 bool rows_copied(const deoct_dataset* ds, const int32_t* idx);
-// whether an evaluation that has no planes is one for the bit-sliced evaluator (api.cu)
-bool slice_once(const deoct_ctx* ctx, int64_t n_sub, int P);
 // The evaluator plan of one population on one (sub)set of a dataset, for the shape `cfg`:
 // rank rows and labels are staged by bulk copies when the set is the whole dataset and the
 // rows are 16-byte aligned (ranks base and row stride), else gathered with plain loads.

@@ -574,7 +574,7 @@ bool level_slice(deoct_ctx* ctx, const deoct_dataset* ds, BatchedEval* be, int P
     e.ptile0 = tiles;
     tiles += slc::slice_tiles(e.count);
   }
-  if (!slc::slice_choose(ctx, Dt, ds->F, ds->K, P, nb, tiles, (int)be->probs.size(), sh)) return false;
+  if (!slc::slice_choose(ctx, ds->rank_bytes, true, Dt, ds->F, ds->K, P, nb, tiles, (int)be->probs.size(), sh)) return false;
   if (!slc::slice_wins(ctx, *sh, ballot)) return false;
   for (EvalProb& e : be->probs) {
     e.nb = nb;
@@ -734,7 +734,7 @@ int de_batched(deoct_ctx* ctx, const deoct_dataset* ds, const Compacted& c, uint
     DEOCT_TRY(scratch_get(ctx, SL_EVAL_PROBS, sizeof(EvalProb) * M, (void**)&dep));
     DEOCT_TRY(build_plan(ctx, &be, scfg, F, K, P, s));
     level_planes(ctx, ds, &be, &sh);
-    if (sh.raw && !slice_once(ctx, nsum_of(c, M), P)) sliced = false;
+    if (sh.raw && !(slc::slice_once(ctx, nsum_of(c, M), P) && slc::slice_wins_once(ctx, sh, ballot))) sliced = false;
   }
   DEOCT_TRY(upload(ctx, SL_EVAL_PROBS, be.probs, &dep, s));
   be.plan.d_probs = dep;

@@ -101,6 +101,7 @@ def test_single_evaluation_of_wide_ranks(F, digits, past):
     th[0] = 0
     th[1] = np.where(a[1] > 0, nu[np.maximum(a[1].astype(int) - 1, 0)] - 1, 0)
     ctx = deoct.Context(0)
+    ctx.set_eval_slicing(1)
     counts, errors = deoct.deoct_eval_population(ctx, ds, to_dev(a.astype(np.uint16)), to_dev(th.astype(np.uint32)), depth)
     got = ctx.slice_stats()
     ref = oracle.eval_counts_omp(ranks, y, K, a, th, depth)

@@ -85,3 +85,27 @@ def test_slicing_mode_is_checked():
         with pytest.raises(deoct.DeoctError):
             ctx.set_eval_slicing(bad)
     ctx.close()
+
+
+@pytest.mark.parametrize("n,F,K,bits,W,P,depth,sliced", [
+    (150_000, 24, 9, 20, 4, 931, 5, False),  # 814 us without planes against 381
+    (480_000, 50, 3, 10, 2, 346, 4, False),  # 470 against 270
+    (1_000_000, 10, 2, 16, 2, 512, 4, True)])
+def test_measured_single_evaluations_take_the_faster_evaluator(n, F, K, bits, W, P, depth, sliced):
+    import torch
+    from paper_2311_06952_gb300 import deoct
+    ds = _ds(n, F, K, bits, W)
+    g = torch.Generator(device="cuda").manual_seed(n)
+    B = (1 << depth) - 1
+    a = torch.randint(0, F + 1, (P, B), generator=g, device="cuda").to(torch.int16)
+    th = torch.randint(0, 1 << bits, (P, B), generator=g, device="cuda", dtype=torch.int32)
+    out = []
+    for mode in (-1, 0, 1):
+        ctx = deoct.Context(0)
+        ctx.set_eval_slicing(mode)
+        counts, errors = deoct.deoct_eval_population(ctx, ds, a, th, depth)
+        out.append((counts, errors, ctx.slice_stats()[0]))
+        ctx.close()
+    assert [o[2] for o in out] == [0, int(sliced), 1]
+    for o in out[1:]:
+        assert torch.equal(o[0], out[0][0]) and torch.equal(o[1], out[0][1])
