@@ -45,12 +45,12 @@ INT32_LANES_PER_SM = 128  # Blackwell SM: 4 partitions x 32 lanes issue INT32
 # taken on: a hash of the bit-sliced evaluator's code (eval_slice.cu, eval_slice.cuh), of
 # the re-laid kernel's and its shape chooser in csrc/eval.cu and of the headers both are
 # built from (eval_kernel.cuh, common.cuh), comments and whitespace left out.
-EVAL_TRAFFIC = {"source_sha256_16": "4c2a85aa0dc07e19", "bytes": 212_132_864 + 3_597_568,
+EVAL_TRAFFIC = {"source_sha256_16": "a91f375849e712f5", "bytes": 205_693_440 + 4_423_680,
                 # the same capture: issue rate (of 4 per SM per cycle), pipe and DRAM figures
-                "ncu": {"inst_per_cycle": 3.4608, "issue_frac": 0.8652, "alu_pipe_frac": 0.8130,
-                        "shared_pipe_frac": 2742440261 / 152 / (10.224672e-3 * 2.07e9),
-                        "inst_per_chunk": 34.23, "dram_gbs": (212_132_864 + 3_597_568) / 10.224672e-3 / 1e9,
-                        "dram_frac_of_peak": (212_132_864 + 3_597_568) / 10.224672e-3 / 1e9 / 6777.3}}
+                "ncu": {"inst_per_cycle": 1.7562, "issue_frac": 0.4390, "alu_pipe_frac": 0.4230,
+                        "shared_pipe_frac": 0.8553, "inst_per_chunk": 6.19,
+                        "dram_gbs": (205_693_440 + 4_423_680) / 3.645472e-3 / 1e9,
+                        "dram_frac_of_peak": (205_693_440 + 4_423_680) / 3.645472e-3 / 1e9 / 6681.5}}
 
 
 def _strip_comments(src):

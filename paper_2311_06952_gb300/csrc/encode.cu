@@ -84,7 +84,8 @@ __global__ void __launch_bounds__(kThreads) keys_kernel(const float* __restrict_
 }
 
 // ---------------------------------------------------------------------------
-// segmented LSD radix sort, one sweep a pass
+// segmented LSD radix sort, one sweep a pass (the published one-sweep form: Adinets and
+// Merrill, 2022, over Merrill and Garland's decoupled look-back, 2016)
 // ---------------------------------------------------------------------------
 // The digit counts of all passes come from one read of the keys (rs_hist_kernel).
 // A pass then reads each key and value once and writes each once: a tile of 4096

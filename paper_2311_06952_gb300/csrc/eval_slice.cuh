@@ -29,7 +29,7 @@
 // 34% slower: fewer registers than the masks of eight leaves need).
 //
 // Measured on GB300, per launch (before: the re-laid kernel, whose warps route 32
-// samples by ballots, 34 instructions per 32 evaluations against 8 here): n = 1e7,
+// samples by ballots, 34 instructions per 32 evaluations against 6.2 here): n = 1e7,
 // F = 10, K = 2, 1024 trees of depth 4, uint16: 10.2 ms -> 3.6 ms; n = 1e6, F = 30,
 // K = 4, 128 trees of depth 3, uint32: 142 -> 86 us; depth 2: 107 -> 55 us; n = 6e4,
 // F = 24, K = 5, 128 trees of depth 3: 23.0 -> 12.6 us; n = 2e6, 256 trees of depth
